@@ -591,7 +591,11 @@ void build_partition(pj_index& idx, int tau, Partition& part) {
                                                            tau, part.scheme, keys.p, part.postings.p);
   PJ_LAUNCHED("k_seg_records");
   trace_mark(c, "partition: records");
-  radix_sort_pairs<unsigned long long>(c, keys.p, part.postings.p, nrec, 64);
+  // the key's used bits: i and l take as many as tau and the longest string
+  // need (two passes of eight fewer for strings below 256 bytes)
+  const unsigned long long used =
+      ~0ull << 32 | ((1ull << bits_for((uint64_t)idx.lmax + 1)) - 1) << 8 | ((1ull << bits_for((uint64_t)tau + 2)) - 1);
+  radix_sort_bits<unsigned long long>(c, keys.p, part.postings.p, nrec, used);
   trace_mark(c, "partition: sort");
 
   DBuf<uint32_t> flags(c, nrec), uidx(c, nrec);

@@ -1641,8 +1641,8 @@ static unsigned long long verify_pair_keys(const Ctx& c, const ProbeView& v, DBu
   const int pshift = bits_for(v.n_index);
   const int nbits = pshift + (SELF ? pshift : bits_for((unsigned long long)v.pbegin + v.pcount));
   DBuf<unsigned long long> k1(c, n_cand);
-  DBuf<uint32_t> v0(c, n_cand), v1(c, n_cand);
-  const bool second = radix_sort_pairs_dn<unsigned long long>(c, k0.p, v0.p, k1.p, v1.p, n_cand, nullptr, nbits);
+  const bool second =
+      radix_sort_pairs_dn<unsigned long long>(c, k0.p, nullptr, k1.p, nullptr, n_cand, nullptr, nbits);
   unsigned long long* sorted = second ? k1.p : k0.p;
   unsigned long long* ukeys = second ? k0.p : k1.p;
   DBuf<uint32_t> flags(c, n_cand), pos(c, n_cand);
@@ -2550,7 +2550,7 @@ struct SelfPlan {
   DBuf<unsigned char> counters, arena;
   DBuf<PlanSizes> sizes;
   DBuf<unsigned long long> nuniq, gmask, hcnt, hoff, pk0, pk1, ukeys, ak0, ak1;
-  DBuf<uint32_t> gcounts, goff, pv0, pv1, pflags, ppos, ae0, ae1, flags, pos;
+  DBuf<uint32_t> gcounts, goff, pflags, ppos, ae0, ae1, flags, pos;
   DBuf<Hit> hits;
   DBuf<pj_pair> out;
   // the fused form: k_fused_self over probes [q_cut, end), the chunked
@@ -2573,7 +2573,7 @@ struct SelfPlan {
                                        &fwork, &fovf, &fhcnt, &fhoff, &fhk, &fz, &fstart};
     for (auto* b : b64) b->release();
     fheavy.release();
-    DBuf<uint32_t>* b32[] = {&gcounts, &goff, &pv0, &pv1, &pflags, &ppos, &ae0, &ae1, &flags, &pos};
+    DBuf<uint32_t>* b32[] = {&gcounts, &goff, &pflags, &ppos, &ae0, &ae1, &flags, &pos};
     for (auto* b : b32) b->release();
     counters.release();
     arena.release();
@@ -2719,7 +2719,7 @@ static void record_self_plan(const Ctx& c, const ProbeView& v, SelfPlan& P) {
       PJ_LAUNCHED("k_pair_keys");
     }
     if (P.fused) record_fused_tail(c, v, P, ctr, sz, acc);  // its pair keys after the chunked ones
-    const bool second = radix_sort_pairs_dn<unsigned long long>(c, P.pk0.p, P.pv0.p, P.pk1.p, P.pv1.p, P.cap_cands,
+    const bool second = radix_sort_pairs_dn<unsigned long long>(c, P.pk0.p, nullptr, P.pk1.p, nullptr, P.cap_cands,
                                                                 &sz->cands, 2 * pshift);
     const unsigned long long* sorted = second ? P.pk1.p : P.pk0.p;
     k_run_heads<<<stride_grid(P.cap_cands), 256, 0, c.stream>>>(sorted, P.cap_cands, P.pflags.p, &sz->cands);
@@ -2822,8 +2822,6 @@ static std::shared_ptr<SelfPlan> make_self_plan(pj_index& idx, const ProbeView& 
   P->hoff.reset(c, P->cap_hits);
   P->pk0.reset(c, P->cap_cands);
   P->pk1.reset(c, P->cap_cands);
-  P->pv0.reset(c, P->cap_cands);
-  P->pv1.reset(c, P->cap_cands);
   P->pflags.reset(c, P->cap_cands);
   P->ppos.reset(c, P->cap_cands);
   P->ukeys.reset(c, P->cap_cands);
@@ -2853,10 +2851,10 @@ static std::shared_ptr<SelfPlan> make_self_plan(pj_index& idx, const ProbeView& 
     P->fz.reset(c, 4);
     P->fstart.reset(c, FOVF_LISTS + 1);
   }
-  size_t arena_bytes = scan_temp_bytes(n_groups, 4) + scan_temp_bytes(P->cap_hits, 8) +
-                       2 * scan_temp_bytes(P->cap_cands, 4) + sort_temp_bytes(P->cap_cands) +
-                       scan_temp_bytes(P->cap_acc, 4) + sort_temp_bytes(P->cap_acc) +
-                       scan_temp_bytes(P->heavy_cap, 8) + (1u << 16);
+  size_t arena_bytes = scan_temp_bytes(n_groups) + scan_temp_bytes(P->cap_hits) +
+                       2 * scan_temp_bytes(P->cap_cands) + sort_temp_bytes(P->cap_cands) +
+                       scan_temp_bytes(P->cap_acc) + sort_temp_bytes(P->cap_acc) +
+                       scan_temp_bytes(P->heavy_cap) + (1u << 16);
   for (int attempt = 0;; ++attempt) {
     P->arena.reset(c, arena_bytes);
     c.sync();

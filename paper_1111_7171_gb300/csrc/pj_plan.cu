@@ -126,8 +126,8 @@ void alloc_pairs(pj_plan& P) {
 // Records the pipeline into a fresh graph and instantiates it.
 void capture(pj_plan& P) {
   P.drop_graph();
-  size_t arena_bytes = scan_temp_bytes(P.d.cap_q, 8) + scan_temp_bytes(P.d.cap_groups, 4) +
-                       scan_temp_bytes(P.d.cap_hits, 8) + scan_temp_bytes(P.d.cap_acc, 4) +
+  size_t arena_bytes = scan_temp_bytes(P.d.cap_q) + scan_temp_bytes(P.d.cap_groups) +
+                       scan_temp_bytes(P.d.cap_hits) + scan_temp_bytes(P.d.cap_acc) +
                        sort_temp_bytes(P.d.cap_acc) + (1u << 16);
   for (int attempt = 0;; ++attempt) {
     P.arena.reset(P.ctx, arena_bytes);

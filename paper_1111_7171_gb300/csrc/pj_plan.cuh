@@ -7,6 +7,7 @@
 #include <string>
 
 #include "pj_internal.cuh"
+#include "pj_prims.cuh"
 #include "pj_probe.cuh"
 
 namespace pj {
@@ -111,22 +112,15 @@ inline void arena_free(void*, void*, void*) {}
 
 inline size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
-// Temporaries of exclusive_scan_dn over n items of es bytes: two arrays of
-// tile sums per level of the recursion.
-inline size_t scan_temp_bytes(size_t n, size_t es) {
-  size_t b = 0;
-  while (n > 4096) {
-    n = (n + 4095) / 4096;
-    b += 2 * align256(n * es);
-  }
-  return b;
+// Temporaries of exclusive_scan_dn over n items: a status word per tile.
+inline size_t scan_temp_bytes(size_t n) {
+  return n <= SCAN_SMALL ? 0 : align256((n + SCAN_TILE - 1) / SCAN_TILE * 8);
 }
 
-// Temporaries of radix_sort_pairs_dn over n items: digit histograms and
-// their offsets (256 per 2048-item tile), and their scan.
+// Temporaries of radix_sort_pairs_dn over n items: the digit counts and, for
+// up to 8 passes, a status word per digit and tile.
 inline size_t sort_temp_bytes(size_t n) {
-  const size_t h = 256 * ((n + 2047) / 2048);
-  return 2 * align256(h * 4) + scan_temp_bytes(h, 4);
+  return align256(8 * (RS_HIST_WORDS + 8 * 256 * ((n + RS_TILE - 1) / RS_TILE)));
 }
 
 // Enqueues the whole query pipeline for the buffers in d on c's stream

@@ -6,6 +6,14 @@
 
 namespace pj {
 
+// Items per tile: the scan's, the single-block scan's, the radix pass's and
+// the single-block sort's; status and histogram words of a sort.
+constexpr size_t SCAN_TILE = 4096;
+constexpr size_t SCAN_SMALL = 16384;
+constexpr size_t RS_TILE = 4096;
+constexpr size_t RSS_TILE = 8192;
+constexpr size_t RS_HIST_WORDS = 8 * 256 / 2;
+
 // out[k] = in[0] + ... + in[k-1] for k < n (out must not alias in).
 template <class T>
 void exclusive_scan(const Ctx& c, const T* in, T* out, size_t n);
@@ -14,6 +22,12 @@ void exclusive_scan(const Ctx& c, const T* in, T* out, size_t n);
 // digits).  Sorted pairs end up in keys/vals.
 template <class K>
 void radix_sort_pairs(const Ctx& c, K* keys, uint32_t* vals, size_t n, int nbits);
+
+// The same by the set bits of `bits`, which has every bit in which two keys
+// may differ (digits start at set bits; bits that are equal in all keys cost
+// no pass).
+template <class K>
+void radix_sort_bits(const Ctx& c, K* keys, uint32_t* vals, size_t n, unsigned long long bits);
 
 // Device-sized forms, for work recorded into a CUDA graph: the launch covers
 // `cap` items and the kernels process the first min(cap, *n_dev) of them
