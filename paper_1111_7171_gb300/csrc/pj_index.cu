@@ -242,6 +242,37 @@ __global__ void k_signatures(const uint8_t* __restrict__ bytes, const uint64_t* 
     bm[k] = char_signature(bytes + off[k], (int)(off[k + 1] - off[k]));
 }
 
+// The bits of any and of all of n bytes: orr and ~andd by atomicOr into
+// out[0], out[1] (zero before).
+__global__ void k_byte_bits(const uint8_t* __restrict__ bytes, uint64_t n, uint32_t* __restrict__ out) {
+  uint32_t any = 0, inv = 0;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) {
+    any |= bytes[k];
+    inv |= ~(uint32_t)bytes[k] & 255u;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    any |= __shfl_xor_sync(FULL, any, o);
+    inv |= __shfl_xor_sync(FULL, inv, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    if (any) atomicOr(out, any);
+    if (inv) atomicOr(out + 1, inv);
+  }
+}
+
+// Bit planes of n strings, one thread each; bits: k_byte_bits' words (NULL:
+// bb holds the bits).
+__global__ void k_planes(const uint8_t* __restrict__ bytes, const uint64_t* __restrict__ off, uint32_t n,
+                         const uint32_t* __restrict__ bits, ByteBits bb, Planes* __restrict__ planes) {
+  if (bits) bb = ByteBits{~bits[1] & 255u, bits[0]};
+  for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+    const uint64_t o = off[k], len = off[k + 1] - o;
+    planes[k] = string_planes(bytes + o, (int)min(len, (uint64_t)PLANE_LEN + 1), bb);
+  }
+}
+
 // Prefix values (seg_value_from_prefix) of n strings: string k's |k| + 1
 // values start at H[off[k] + k].  One warp per string, 32 bytes per step:
 // each byte is the affine map h -> h * SEG_B + byte, and a shuffle scan
@@ -327,11 +358,7 @@ __global__ void k_side_sigs(const uint8_t* __restrict__ sbytes, const uint64_t* 
     for (int i = 1; i <= tau + 1; ++i) {  // prefixes: bytes [0, P_i)
       int P, li;
       segment_m(l, tau + 1, 0, scheme, i, P, li);
-      for (; k < P; ++k) {
-        const int sh = 4 * (int)(s[k] % SIDE_BUCKETS);
-        const unsigned long long field = (t >> sh) & 15ull;
-        if (field != 15ull) t |= (field + 1ull) << sh;
-      }
+      for (; k < P; ++k) side_count(t, s[k]);
       out[i - 1].x = t;
     }
     t = 0;
@@ -339,11 +366,7 @@ __global__ void k_side_sigs(const uint8_t* __restrict__ sbytes, const uint64_t* 
     for (int i = tau + 1; i >= 1; --i) {  // suffixes: bytes [P_i + l_i, l)
       int P, li;
       segment_m(l, tau + 1, 0, scheme, i, P, li);
-      for (; k > P + li; --k) {
-        const int sh = 4 * (int)(s[k - 1] % SIDE_BUCKETS);
-        const unsigned long long field = (t >> sh) & 15ull;
-        if (field != 15ull) t |= (field + 1ull) << sh;
-      }
+      for (; k > P + li; --k) side_count(t, s[k - 1]);
       out[i - 1].y = t;
     }
   }
@@ -358,12 +381,12 @@ __global__ void k_post_records(const uint32_t* __restrict__ postings, const unsi
   for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t sid = postings[k];
     if (!sides) {
-      recs[k] = make_rec(sid, 0ull, 0ull);
+      recs[k] = make_rec(sid, SidePair{{0u, 0u, 0u}});
       continue;
     }
     const int i = (int)(keys[k] & 0xFFu);
     const ulonglong2 sd = sides[(uint64_t)(sid - first) * (tau + 1) + i - 1];
-    recs[k] = make_rec(sid, sd.x, sd.y);
+    recs[k] = make_rec(sid, side_pair(sd.x, sd.y));
   }
 }
 
@@ -439,6 +462,10 @@ static void stage_strings(const Ctx& c, const pj_strings& S, DBuf<uint8_t>& byte
   *total = tot;
 }
 
+// Average length up to which strings get bit planes (most are then at most
+// PLANE_LEN long).
+constexpr uint64_t PLANES_MAX_AVG_LEN = 24;
+
 void build_store(pj_index& idx, const pj_strings& S) {
   const Ctx& c = idx.ctx;
   const uint32_t n = S.n;
@@ -513,6 +540,21 @@ void build_store(pj_index& idx, const pj_strings& S) {
                                                                                 idx.sref.p);
     PJ_LAUNCHED("k_refs");
   }
+  // Bit planes for short strings, 32 bytes each (not under a device budget:
+  // they are only for speed).
+  DBuf<uint32_t> bits;
+  const bool planes = n && !c.budget && total <= PLANES_MAX_AVG_LEN * n;
+  if (planes) {
+    bits.reset(c, 2);
+    PJ_CUDA(cudaMemsetAsync(bits.p, 0, 2 * sizeof(uint32_t), c.stream));
+    idx.splanes.reset(c, n);
+    k_byte_bits<<<std::min<unsigned>(ceil_div(total ? total : 1, 256 * 16), sm_grid_cap(8)), 256, 0, c.stream>>>(
+        idx.sbytes.p, total, bits.p);
+    PJ_LAUNCHED("k_byte_bits");
+    k_planes<<<std::min<unsigned>(ceil_div(n, 128), sm_grid_cap(16)), 128, 0, c.stream>>>(
+        idx.sbytes.p, idx.soff.p, n, bits.p, ByteBits{0, 0}, idx.splanes.p);
+    PJ_LAUNCHED("k_planes");
+  }
   idx.sph.reset(c, (size_t)total + n + 1);
   if (n) {
     const unsigned blocks = std::min<unsigned>(ceil_div((size_t)n * 32, 256), sm_grid_cap(16));
@@ -526,7 +568,10 @@ void build_store(pj_index& idx, const pj_strings& S) {
   idx.h_bbeg.resize((size_t)idx.lmax + 2);
   PJ_CUDA(cudaMemcpyAsync(idx.h_bbeg.data(), idx.bbeg.p, idx.h_bbeg.size() * sizeof(uint32_t),
                           cudaMemcpyDeviceToHost, c.stream));
+  uint32_t h_bits[2] = {0, 0};
+  if (planes) PJ_CUDA(cudaMemcpyAsync(h_bits, bits.p, sizeof(h_bits), cudaMemcpyDeviceToHost, c.stream));
   c.sync();
+  idx.byte_bits = ByteBits{~h_bits[1] & 255u, h_bits[0]};
 }
 
 // Average indexed length above which a table gets 2 presence-bitmap bytes
@@ -719,7 +764,7 @@ Partition& ensure_partition(pj_index& idx, int tau, float* ms) {
   return part;
 }
 
-void upload_probe_set(const Ctx& c, const pj_strings& R, ProbeSet& out) {
+void upload_probe_set(const Ctx& c, const pj_index& idx, const pj_strings& R, ProbeSet& out, bool planes) {
   const uint8_t* dbytes = nullptr;
   const uint64_t* doff = nullptr;
   uint64_t total = 0;
@@ -749,6 +794,12 @@ void upload_probe_set(const Ctx& c, const pj_strings& R, ProbeSet& out) {
   if (R.n) {
     k_signatures<<<std::min<unsigned>(ceil_div(R.n, 256), sm_grid_cap(8)), 256, 0, c.stream>>>(dbytes, doff, R.n, out.bm.p);
     PJ_LAUNCHED("k_signatures");
+    if (planes && idx.splanes.p) {
+      out.planes.reset(c, R.n);
+      k_planes<<<std::min<unsigned>(ceil_div(R.n, 128), sm_grid_cap(16)), 128, 0, c.stream>>>(
+          dbytes, doff, R.n, nullptr, idx.byte_bits, out.planes.p);
+      PJ_LAUNCHED("k_planes");
+    }
   }
   out.bytes = dbytes;
   out.off = doff;
@@ -762,7 +813,7 @@ void upload_probe_set(const Ctx& c, const pj_strings& R, ProbeSet& out) {
 
 uint64_t pj_index::device_bytes() const {
   uint64_t b = sbytes.bytes() + soff.bytes() + slen.bytes() + perm.bytes() + bbeg.bytes() + sbm.bytes() + sph.bytes() +
-               sref.bytes();
+               sref.bytes() + splanes.bytes();
   for (const auto& p : parts)
     b += p.table.bytes() + p.fp.bytes() + p.postings.bytes() + p.precs.bytes() + p.gorder[0].bytes() +
          p.gorder[1].bytes();

@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "pj_common.cuh"
+#include "pj_verify.cuh"
 
 namespace pj {
 
@@ -373,19 +374,23 @@ __host__ __device__ __forceinline__ int table_find(const Slot* __restrict__ t, c
 // the parts right of them.  The character-count bound above holds for each
 // side on its own, with thresholds that add up to tau, so testing the two
 // sides rejects far more matches than testing the whole strings.  A side
-// signature is a 48-bit thermometer code: characters fall into SIDE_BUCKETS
-// = 12 buckets (c mod 12), bucket b owns bits 4b .. 4b+3, of which the lowest
-// min(count_b, 4) are set; the bound of two sides is the larger of the two
-// popcounts of x & ~y and y & ~x.
+// signature is the side's character counts, 4 bits each: characters fall
+// into SIDE_BUCKETS = 12 buckets (c mod 12), bucket b owns bits 4b .. 4b+3
+// and holds min(count_b, 15).  With L1 the sum of the counts' differences and
+// D the difference of the lengths, a substitution changes L1 by at most 2 and
+// an insertion or deletion changes L1 and D by at most 1, so 2 ED(x, y) >= L1
+// + |D| (a capped count differs no more than the count itself).
 constexpr int SIDE_BUCKETS = 12;
+constexpr uint32_t SIDE_MASK = 0x0F0F0F0Fu;
+
+__host__ __device__ __forceinline__ void side_count(unsigned long long& t, uint8_t c) {
+  const int sh = 4 * (int)(c % SIDE_BUCKETS);
+  if (((t >> sh) & 15ull) != 15ull) t += 1ull << sh;
+}
 
 __host__ __device__ __forceinline__ unsigned long long side_signature(const uint8_t* p, int n) {
   unsigned long long t = 0;
-  for (int k = 0; k < n; ++k) {
-    const int sh = 4 * (int)(p[k] % SIDE_BUCKETS);
-    const unsigned long long field = (t >> sh) & 15ull;  // 0, 1, 3, 7 or 15
-    if (field != 15ull) t |= (field + 1ull) << sh;       // set the next bit
-  }
+  for (int k = 0; k < n; ++k) side_count(t, p[k]);
   return t;
 }
 
@@ -397,36 +402,118 @@ __host__ __device__ __forceinline__ int popcount64(unsigned long long x) {
 #endif
 }
 
+// acc + the sum of the four bytes' absolute differences (one instruction:
+// about 2 cycles per warp here, against 8.8 for a popcount).
+__host__ __device__ __forceinline__ unsigned byte_distance(uint32_t x, uint32_t y, unsigned acc) {
+#ifdef __CUDA_ARCH__
+  return __vsadu4(x, y) + acc;
+#else
+  for (int k = 0; k < 32; k += 8) {
+    const int a = (int)(x >> k & 255u), b = (int)(y >> k & 255u);
+    acc += (unsigned)(a > b ? a - b : b - a);
+  }
+  return acc;
+#endif
+}
+
+// The two signatures of a match or a posting in 3 words: byte j of word k
+// holds bucket 4k + j, the left side's count in its low four bits and the
+// right side's in its high four, so that each side's counts come out as bytes
+// by one mask.
+struct SidePair {
+  uint32_t w[3];
+};
+
+__host__ __device__ __forceinline__ SidePair side_pair(unsigned long long left, unsigned long long right) {
+  SidePair s;
+  for (int k = 0; k < 3; ++k) {
+    uint32_t w = 0;
+    for (int j = 0; j < 4; ++j) {
+      const int sh = 4 * (4 * k + j);
+      w |= (uint32_t)(left >> sh & 15ull) << (8 * j) | (uint32_t)(right >> sh & 15ull) << (8 * j + 4);
+    }
+    s.w[k] = w;
+  }
+  return s;
+}
+
+// The sums of the counts' differences of the left and the right sides.
+__host__ __device__ __forceinline__ void side_distances(const SidePair& x, const SidePair& y, unsigned& left,
+                                                        unsigned& right) {
+  left = right = 0;
+  for (int k = 0; k < 3; ++k) {
+    left = byte_distance(x.w[k] & SIDE_MASK, y.w[k] & SIDE_MASK, left);
+    right = byte_distance(x.w[k] >> 4 & SIDE_MASK, y.w[k] >> 4 & SIDE_MASK, right);
+  }
+}
+
+// The bound from the counts alone (no lengths): ED >= max over the two
+// directions of the summed surplus.
 __host__ __device__ __forceinline__ int side_bound(unsigned long long x, unsigned long long y) {
-  const int a = popcount64(x & ~y), b = popcount64(y & ~x);
+  int a = 0, b = 0;
+  for (int sh = 0; sh < 4 * SIDE_BUCKETS; sh += 4) {
+    const int d = (int)(x >> sh & 15ull) - (int)(y >> sh & 15ull);
+    if (d > 0) a += d; else b -= d;
+  }
   return a > b ? a : b;
 }
 
 // What the screen in front of extension verification needs about one
 // posting, stored beside the postings in the same order so that the
 // candidates of a run are read as one coalesced 16-byte stream: the sid and
-// the side signatures of the indexed string around the posting's segment
-// (48 bits left of it in w[0] and the low half of w[1], 48 bits right of it
-// in the high half of w[1] and w[2]).
+// the side signatures of the indexed string around the posting's segment.
 struct __align__(16) PostRec {
   uint32_t sid;
-  uint32_t w[3];
+  SidePair sides;
 };
 
 __host__ __device__ __forceinline__ uint32_t rec_sid(const PostRec& r) { return r.sid; }
-__host__ __device__ __forceinline__ unsigned long long rec_left(const PostRec& r) {
-  return (unsigned long long)r.w[0] | ((unsigned long long)(r.w[1] & 0xFFFFu) << 32);
-}
-__host__ __device__ __forceinline__ unsigned long long rec_right(const PostRec& r) {
-  return (unsigned long long)(r.w[1] >> 16) | ((unsigned long long)r.w[2] << 16);
-}
-__host__ __device__ __forceinline__ PostRec make_rec(uint32_t sid, unsigned long long left, unsigned long long right) {
+__host__ __device__ __forceinline__ PostRec make_rec(uint32_t sid, const SidePair& sides) {
   PostRec r;
   r.sid = sid;
-  r.w[0] = (uint32_t)left;
-  r.w[1] = (uint32_t)((left >> 32) & 0xFFFFu) | (uint32_t)((right & 0xFFFFu) << 16);
-  r.w[2] = (uint32_t)(right >> 16);
+  r.sides = sides;
   return r;
+}
+
+// A short string in bit planes, for verification without byte loads: bit k
+// of plane b is the b-th of the bits of character k in which the characters of
+// the indexed strings differ (at most 8).  A character that differs from
+// them in another bit equals none of them; where a plane is left, it marks
+// these characters (probes only).  Strings longer than PLANE_LEN keep zeros.
+struct __align__(16) Planes {
+  uint32_t w[8];
+};
+
+// The bits of any of n bytes (orr) and of all of them (andd).
+struct ByteBits {
+  uint32_t andd, orr;
+};
+
+__host__ __device__ __forceinline__ Planes string_planes(const uint8_t* p, int n, ByteBits bb) {
+  Planes t = {{0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u}};
+  if (n > PLANE_LEN) return t;
+  const uint32_t vary = bb.orr & ~bb.andd & 255u, same = ~vary & 255u;
+  for (int k = 0; k < n; ++k) {
+    const uint32_t c = p[k];
+    uint32_t v = vary;
+    bool foreign = ((c ^ bb.andd) & same) != 0;
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      const uint32_t low = v & (0u - v);
+      if (low ? (c & low) != 0 : foreign) t.w[b] |= 1u << k;
+      foreign = low ? foreign : false;  // one plane marks it
+      v &= v - 1;
+    }
+  }
+  return t;
+}
+
+// Planes in use: those of the differing bits and, for probes that are not
+// indexed strings, the marking one.
+__host__ __device__ __forceinline__ int planes_used(ByteBits bb, bool self) {
+  const uint32_t vary = bb.orr & ~bb.andd & 255u;
+  const int n = popcount32(vary);
+  return self || n == 8 ? n : n + 1;
 }
 
 // One threshold's segment index.
@@ -477,6 +564,8 @@ struct pj_index {
   pj::DBuf<pj::Sig> sbm;     // character signatures by sid (char_signature)
   pj::DBuf<uint32_t> sph;    // prefix values (seg_value_from_prefix) by sid, |s| + 1 from soff[sid] + sid
   pj::DBuf<unsigned long long> sref;  // soff[sid] << 16 | slen[sid] by sid
+  pj::DBuf<pj::Planes> splanes;       // bit planes by sid (empty: long strings, or under a device budget)
+  pj::ByteBits byte_bits{0, 0};       // bits of the indexed characters (with splanes)
   std::vector<uint32_t> h_bbeg;
   std::vector<pj::Partition> parts;  // index = tau
   uint64_t device_bytes() const;
@@ -500,10 +589,12 @@ struct ProbeSet {
   const uint64_t* off = nullptr;
   DBuf<uint32_t> len;
   DBuf<Sig> bm;  // character signatures
+  DBuf<Planes> planes;  // bit planes (when the index has them)
   uint32_t n = 0;
   int lmax = 0;
 };
-void upload_probe_set(const Ctx& c, const pj_strings& R, ProbeSet& out);
+// planes: with bit planes if idx has them.
+void upload_probe_set(const Ctx& c, const pj_index& idx, const pj_strings& R, ProbeSet& out, bool planes = true);
 
 // R != S probe of a resident index where probe q has threshold h_tau[q]
 // (host array).  Every threshold present must be built.  Work is ordered on

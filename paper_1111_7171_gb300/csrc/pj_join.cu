@@ -264,10 +264,10 @@ __global__ void __launch_bounds__(BLOCK) k_group_hits(const ProbeView v, unsigne
         uint32_t b;
         const uint32_t c = lookup_key(vt, SELF, q, ls, l, seg_key(s + p, li, l, i), b, err);
         if (c) {
-          Hit hh{q, b, c, (uint32_t)p | ((uint32_t)i << 16) | tau_tag, 0ull, 0ull};
+          Hit hh{q, b, c, (uint32_t)p | ((uint32_t)i << 16) | tau_tag, {{0u, 0u, 0u}}, 0u};
           if (vt.hit_sides) {
-            hh.sl = side_signature(s, p);
-            hh.sr = side_signature(s + p + li, ls - p - li);
+            hh.sides = side_pair(side_signature(s, p), side_signature(s + p + li, ls - p - li));
+            hh.lim = hit_limits(vt.tau, i, ls, l, p, P, li);
           }
           hits[pos++] = hh;
         }
@@ -399,15 +399,21 @@ constexpr int Q_BLOCK = 256;
 constexpr int Q_WARPS = Q_BLOCK / 32;
 constexpr int S_RUN = 8;                 // candidates one lane screens per step
 constexpr int Q_CAP = 32 * S_RUN + 32;   // < 32 left + up to 32 * S_RUN new
-constexpr unsigned long long Q_CHUNK = 8ull * 32 * S_RUN;  // candidates a warp takes at a time (at least)
+constexpr int Q_SECOND = 64;             // < 32 left + up to 32 new
+constexpr unsigned long long Q_CHUNK = 8ull * 32 * S_RUN;  // candidates a warp takes at a time
+constexpr unsigned long long Q_CHUNK_MIN = 128;            // ... in launches too small to fill the warps
 
-// Chunk of a queued verification launch over n candidates on `grid` blocks:
+// Chunk of a queued verification launch over n candidates by n_warps warps:
 // Q_CHUNK, times up to 4 when every warp gets at least 512 chunks of that
 // size (measured on 2.2e10 candidates: 3% less time with 4; on 3e8, where a
-// warp gets 30 chunks, larger chunks unbalance the warps).
-static unsigned long long queued_chunk(unsigned long long n, unsigned grid) {
-  const unsigned long long per_warp = n / ((unsigned long long)grid * Q_WARPS * Q_CHUNK);
-  return Q_CHUNK * std::min<unsigned long long>(4, std::max<unsigned long long>(1, per_warp / 512));
+// warp gets 30 chunks, larger chunks unbalance the warps), and in launches
+// that have less than a chunk for every warp an even share, so that a small
+// batch does not leave most of the GPU idle (64 queries: 162 -> 45 us).
+__host__ __device__ __forceinline__ unsigned long long queued_chunk(unsigned long long n, unsigned long long n_warps) {
+  const unsigned long long share = n / n_warps;
+  if (share >= 512 * Q_CHUNK) return Q_CHUNK * ::min(4ull, share / (512 * Q_CHUNK));
+  if (share >= Q_CHUNK) return Q_CHUNK;
+  return ::max(Q_CHUNK_MIN, (share + 31) / 32 * 32);
 }
 
 // One lane's hit: index h, its posting for candidate c is rec_base + c
@@ -415,8 +421,8 @@ static unsigned long long queued_chunk(unsigned long long n, unsigned grid) {
 struct LaneHit {
   uint32_t h;
   uint32_t rec_base;
-  uint32_t q, pi;
-  unsigned long long sl, sr;  // the probe's side signatures around the match
+  uint32_t q, pi, lim;
+  SidePair sides;  // the probe's side signatures around the match
 };
 
 __device__ __forceinline__ void lane_hit_set(const Hit* __restrict__ hits, uint32_t h, unsigned long long c_lo,
@@ -426,8 +432,8 @@ __device__ __forceinline__ void lane_hit_set(const Hit* __restrict__ hits, uint3
   lh.rec_base = hit.begin - (uint32_t)c_lo;
   lh.q = hit.q;
   lh.pi = hit.pi;
-  lh.sl = hit.sl;
-  lh.sr = hit.sr;
+  lh.lim = hit.lim;
+  lh.sides = hit.sides;
 }
 
 // Extension verification of one queue entry: probe q, indexed sid r, and
@@ -460,6 +466,90 @@ __device__ __forceinline__ void verify_queued_entry(const ProbeView& v, uint32_t
   }
 }
 
+// A warp's queues in shared memory.  A screened match waits in the first
+// until 32 of them are verified together; with bit planes (short strings, tau
+// <= 4) that is only the side with the smaller threshold, and the matches
+// whose first side passed (its distance in place of the left limit) wait in
+// the second until 32 of them can have the other side verified: most matches
+// fail on the first side, and lanes with nothing left to do would idle through
+// the second side's wider band.
+struct SecondQueue {
+  uint32_t q[Q_SECOND], sid[Q_SECOND], pi[Q_SECOND], lim[Q_SECOND];
+};
+struct QueueWarp {
+  uint32_t q[Q_CAP], sid[Q_CAP], pi[Q_CAP], lim[Q_CAP];
+  SecondQueue second;
+};
+
+// First side of one match per lane (`in` lanes have one).  Matches without
+// planes (lengths 0 in lim) are verified as a whole.  n2: the second queue's
+// size, the same in every lane.
+template <int MAXW, bool SELF, bool MULTI>
+__device__ __forceinline__ void verify_first(const ProbeView& v, SecondQueue& w, bool in, uint32_t q, uint32_t r,
+                                             uint32_t pi, uint32_t lim, int& n2, AccOut out, Counters* ctr,
+                                             unsigned long long& cells) {
+  bool pass = false;
+  uint32_t d1 = 0;
+  if (in) {
+    if (MAXW <= 5 && v.pplanes && lim >> 16) {
+      const ProbeView vt = MULTI ? view_for_tau(v, (int)(pi >> 24)) : v;
+      const PlaneMatch m = plane_match(vt, q, r, pi, lim);
+      const int tl = m.i - 1, tr = m.tau + 1 - m.i;
+      unsigned c = 0;
+      if (m.li <= SEG_EXACT_MAX || plane_segment(m)) {
+        const bool right = tr < tl;
+        d1 = (uint32_t)plane_side<(MAXW - 1) / 2>(m, right, c);
+        pass = (int)d1 <= (right ? tr : tl);
+      }
+      cells += c;
+    } else {
+      verify_queued_entry<MAXW, SELF, MULTI>(v, q, r, pi, out, ctr, cells);
+    }
+  }
+  if (MAXW <= 5) {
+    __syncwarp();
+    const unsigned b = __ballot_sync(FULL, pass);
+    if (pass) {
+      const int slot = n2 + __popc(b & lanemask_lt());
+      w.q[slot] = q;
+      w.sid[slot] = r;
+      w.pi[slot] = pi;
+      w.lim[slot] = (lim & ~0xFFu) | d1;
+    }
+    n2 += __popc(b);
+    __syncwarp();
+  }
+}
+
+// Second side of the second queue's last min(n2, 32) entries.
+template <int MAXW, bool SELF, bool MULTI>
+__device__ __forceinline__ void verify_second(const ProbeView& v, SecondQueue& w, int& n2, AccOut out, Counters* ctr,
+                                              unsigned long long& cells) {
+  const int lane = (int)(threadIdx.x & 31u);
+  const int n = ::min(n2, 32);
+  n2 -= n;
+  const int e = n2 + (lane < n ? lane : 0);
+  const uint32_t q = w.q[e], r = w.sid[e], pi = w.pi[e], lim = w.lim[e];
+  __syncwarp();  // taken before any later write
+  if (lane < n) {
+    const ProbeView vt = MULTI ? view_for_tau(v, (int)(pi >> 24)) : v;
+    const PlaneMatch m = plane_match(vt, q, r, pi, lim);
+    const int tl = m.i - 1, tr = m.tau + 1 - m.i;
+    const bool right = !(tr < tl);
+    unsigned c = 0;
+    const int d2 = plane_side<MAXW - 1>(m, right, c);
+    cells += c;
+    if (d2 <= (right ? tr : tl)) {
+      const unsigned long long pos = atomicAdd(&ctr->accepted, 1ull);
+      if (pos < out.cap) {
+        out.key[pos] = match_key(v, SELF, q, r);
+        out.ed[pos] = (lim & 0xFFu) + (uint32_t)d2;
+      }
+    }
+  }
+}
+
+// chunk: candidates a warp takes at a time (0: from the device's count).
 template <int MAXW, bool SELF, bool MULTI>
 __global__ void __launch_bounds__(Q_BLOCK) k_verify_queued(const ProbeView v, const Hit* __restrict__ hits,
                                                             const unsigned long long* __restrict__ cand_off,
@@ -467,20 +557,20 @@ __global__ void __launch_bounds__(Q_BLOCK) k_verify_queued(const ProbeView v, co
                                                             unsigned long long n_cand, AccOut out, Counters* ctr,
                                                             const unsigned long long* __restrict__ dn,
                                                             unsigned long long chunk) {
-  __shared__ uint32_t q_q[Q_WARPS][Q_CAP];
-  __shared__ uint32_t q_sid[Q_WARPS][Q_CAP];
-  __shared__ uint32_t q_pi[Q_WARPS][Q_CAP];
+  __shared__ QueueWarp queues[Q_WARPS];
   if (dn) {
     n_hits = min(n_hits, dn[0]);
     n_cand = dn[1];
   }
   unsigned long long cells = 0, filtered = 0;
   int err = 0;
-  const unsigned lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
+  const unsigned lane = threadIdx.x & 31u;
+  QueueWarp& w = queues[threadIdx.x >> 5];
   const unsigned long long warp = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const unsigned long long n_warps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
+  if (chunk == 0) chunk = queued_chunk(n_cand, n_warps);
   const unsigned long long span = 32ull * S_RUN;
-  int qn = 0;  // the same in every lane
+  int qn = 0, n2 = 0;  // the same in every lane
   LaneHit lh;
   lh.h = UINT32_MAX;
   // chunks of `chunk` candidates, dealt to the warps round robin
@@ -497,7 +587,7 @@ __global__ void __launch_bounds__(Q_BLOCK) k_verify_queued(const ProbeView v, co
     }
     for (unsigned long long base = r0; base < r1; base += span) {
       // screen; each survivor goes straight into the queue (one ballot per 32)
-#pragma unroll
+#pragma unroll 2
       for (int k = 0; k < S_RUN; ++k) {
         const unsigned long long c0 = base + 32ull * k;
         if (c0 >= r1) break;  // the same in every lane
@@ -514,45 +604,345 @@ __global__ void __launch_bounds__(Q_BLOCK) k_verify_queued(const ProbeView v, co
             } while (c >= l_hi);
             lane_hit_set(hits, (uint32_t)h, lo, lh);
           }
-          const ProbeView vt = MULTI ? view_for_tau(v, (int)(lh.pi >> 24)) : v;
-          const PostRec rec = vt.precs[lh.rec_base + (uint32_t)c];
+          const PostRec* precs = MULTI ? v.parts[lh.pi >> 24].precs : v.precs;
+          const PostRec rec = precs[lh.rec_base + (uint32_t)c];
           r = rec_sid(rec);
-          if (r >= vt.n_index) {
+          if (r >= v.n_index) {
             err |= 1;
           } else if (!(SELF && r == lh.q)) {
-            // the side bounds against the two sides' thresholds i - 1 and tau + 1 - i
-            const int i = (int)((lh.pi >> 16) & 0xFFu);
-            if (v.pbm && v.hit_sides && (side_bound(lh.sl, rec_left(rec)) > i - 1 ||
-                          side_bound(lh.sr, rec_right(rec)) > vt.tau + 1 - i))
-              ++filtered;
-            else
-              pass = true;
+            // the sides' counts against what their thresholds leave
+            unsigned dl = 0, dr = 0;
+            if (v.hit_sides) side_distances(lh.sides, rec.sides, dl, dr);
+            pass = !v.hit_sides || (dl <= (lh.lim & 0xFFu) && dr <= (lh.lim >> 8 & 0xFFu));
+            if (!pass) ++filtered;
           }
         }
         const unsigned b = __ballot_sync(FULL, pass);
         if (pass) {
           const int slot = qn + __popc(b & lanemask_lt());
-          q_q[wib][slot] = lh.q;
-          q_sid[wib][slot] = r;
-          q_pi[wib][slot] = lh.pi;
+          w.q[slot] = lh.q;
+          w.sid[slot] = r;
+          w.pi[slot] = lh.pi;
+          w.lim[slot] = lh.lim;
         }
         qn += __popc(b);
       }
       __syncwarp();
       while (qn >= 32) {  // the same in every lane
         qn -= 32;
-        const uint32_t q2 = q_q[wib][qn + lane], r2 = q_sid[wib][qn + lane], p2 = q_pi[wib][qn + lane];
-        __syncwarp();  // taken before any later write
-        verify_queued_entry<MAXW, SELF, MULTI>(v, q2, r2, p2, out, ctr, cells);
+        const int e = qn + (int)lane;
+        verify_first<MAXW, SELF, MULTI>(v, w.second, true, w.q[e], w.sid[e], w.pi[e], w.lim[e], n2, out, ctr, cells);
+        if (MAXW <= 5 && n2 >= 32) verify_second<MAXW, SELF, MULTI>(v, w.second, n2, out, ctr, cells);
       }
+      __syncwarp();  // the entries were taken before the next step writes
     }
   }
   __syncwarp();
-  if ((int)lane < qn) verify_queued_entry<MAXW, SELF, MULTI>(v, q_q[wib][lane], q_sid[wib][lane], q_pi[wib][lane],
-                                                             out, ctr, cells);
+  if (qn) {
+    const int e = (int)lane < qn ? (int)lane : 0;
+    verify_first<MAXW, SELF, MULTI>(v, w.second, (int)lane < qn, w.q[e], w.sid[e], w.pi[e], w.lim[e], n2, out, ctr,
+                                    cells);
+  }
+  if (MAXW <= 5) {
+    while (n2) verify_second<MAXW, SELF, MULTI>(v, w.second, n2, out, ctr, cells);
+  }
   add_counter(&ctr->cells, cells);
   add_counter(&ctr->filtered, filtered);
   if (err) atomicOr(&ctr->err, (unsigned long long)err);
+}
+
+// ------------------------------------------- A6, run-major verification --
+//
+// A join of many probes hits the same posting runs again and again, and the
+// queued kernel then spends most of its time on what does not depend on the
+// pair: finding each candidate's hit and loading and unpacking its posting
+// record.  Here the hits are grouped by run first, and a warp of the screen
+// (k_screen_tiles) takes a tile: up to TILE_POSTS postings of one run, whose
+// side counts stay unpacked in registers, against up to TILE_HITS of the
+// run's hits, one after another, each the same for all lanes.  What is left
+// per candidate is six byte distances, three compares and a ballot.  The
+// survivors, (hit, sid), go to a list in device memory, which the
+// verification kernel (k_verify_list) reads 32 at a time: the screen keeps a
+// small loop without divergence, and the verification all its lanes.
+constexpr int TILE_J = 4;                  // postings a lane holds
+constexpr uint32_t TILE_POSTS = 32 * TILE_J;
+constexpr uint32_t TILE_HITS = 256;
+constexpr int T_BLOCK = 256;
+constexpr int T_FLUSH = 128;               // survivors a warp writes out at a time
+constexpr int T_CAP = 32 * TILE_J + T_FLUSH;
+constexpr uint32_t NO_HIT = 0xFFFFFFFFu;   // list entries that hold no survivor
+
+struct __align__(16) Tile {
+  uint32_t post;       // first posting
+  uint32_t posts;      // tiles of the run's postings before it << 8 | postings (1 .. TILE_POSTS) of the tile
+  uint32_t hit, hits;  // the hits
+};
+
+// Hits per run (cnt, by the run's first posting), each hit's rank among them,
+// and the longest of their counts; totals[0] the candidates.
+__global__ void __launch_bounds__(BLOCK) k_run_count(const Hit* __restrict__ hits, unsigned long long n,
+                                                     uint32_t* __restrict__ cnt, uint32_t* __restrict__ longest,
+                                                     uint32_t* __restrict__ rank, unsigned long long* totals) {
+  unsigned long long cand = 0;
+  for (unsigned long long h = (unsigned long long)blockIdx.x * BLOCK + threadIdx.x; h < n;
+       h += (unsigned long long)gridDim.x * BLOCK) {
+    const uint4 a = *reinterpret_cast<const uint4*>(hits + h);  // q, begin, count, pi
+    rank[h] = atomicAdd(&cnt[a.y], 1u);
+    if (longest[a.y] < a.z) atomicMax(&longest[a.y], a.z);
+    cand += a.z;
+  }
+  cand = warp_sum(cand);
+  if ((threadIdx.x & 31) == 0) add_counter(totals, cand);
+}
+
+__global__ void __launch_bounds__(BLOCK) k_run_scatter(const Hit* __restrict__ hits, unsigned long long n,
+                                                       const uint32_t* __restrict__ off,
+                                                       const uint32_t* __restrict__ rank, Hit* __restrict__ out) {
+  for (unsigned long long h = (unsigned long long)blockIdx.x * BLOCK + threadIdx.x; h < n;
+       h += (unsigned long long)gridDim.x * BLOCK) {
+    const uint4* in = reinterpret_cast<const uint4*>(hits + h);
+    const uint4 a = in[0], b = in[1];
+    uint4* o = reinterpret_cast<uint4*>(out + off[a.y] + rank[h]);
+    o[0] = a;
+    o[1] = b;
+  }
+}
+
+__device__ __forceinline__ unsigned long long run_tiles(uint32_t hits, uint32_t posts) {
+  return ((hits + (unsigned long long)TILE_HITS - 1) / TILE_HITS) *
+         ((posts + (unsigned long long)TILE_POSTS - 1) / TILE_POSTS);
+}
+
+// totals[1]: the tiles of all runs.
+__global__ void __launch_bounds__(BLOCK) k_tile_count(const uint32_t* __restrict__ cnt,
+                                                      const uint32_t* __restrict__ longest, unsigned long long n,
+                                                      unsigned long long* totals) {
+  unsigned long long t = 0;
+  for (unsigned long long b = (unsigned long long)blockIdx.x * BLOCK + threadIdx.x; b < n;
+       b += (unsigned long long)gridDim.x * BLOCK)
+    if (cnt[b]) t += run_tiles(cnt[b], longest[b]);
+  t = warp_sum(t);
+  if ((threadIdx.x & 31) == 0) add_counter(totals + 1, t);
+}
+
+// The tiles, in no particular order (totals[2] counts them).
+__global__ void __launch_bounds__(BLOCK) k_tile_emit(const uint32_t* __restrict__ cnt,
+                                                     const uint32_t* __restrict__ longest,
+                                                     const uint32_t* __restrict__ off, unsigned long long n,
+                                                     Tile* __restrict__ tiles, unsigned long long n_tiles,
+                                                     unsigned long long* totals) {
+  const unsigned lane = threadIdx.x & 31u;
+  const unsigned long long stride = (unsigned long long)gridDim.x * BLOCK;
+  for (unsigned long long b0 = (unsigned long long)blockIdx.x * BLOCK + (threadIdx.x & ~31u); b0 < n; b0 += stride) {
+    const unsigned long long b = b0 + lane;
+    const uint32_t c = b < n ? cnt[b] : 0u;
+    const uint32_t m = c ? longest[b] : 0u;
+    const unsigned long long t = c ? run_tiles(c, m) : 0ull;
+    const unsigned long long incl = warp_incl_scan(t);
+    unsigned long long at = 0;
+    if (lane == 31 && incl) at = atomicAdd(totals + 2, incl);
+    at = __shfl_sync(FULL, at, 31) + incl - t;
+    if (t) {
+      const uint32_t h0 = off[b];
+      for (unsigned long long p = 0; p < m; p += TILE_POSTS)
+        for (unsigned long long h = 0; h < c; h += TILE_HITS, ++at)
+          if (at < n_tiles)
+            tiles[at] = Tile{(uint32_t)(b + p), (uint32_t)(p / TILE_POSTS) << 8 | ::min(m - (uint32_t)p, TILE_POSTS),
+                             h0 + (uint32_t)h, ::min(c - (uint32_t)h, TILE_HITS)};
+    }
+  }
+}
+
+// What the screen and the verification of one tile range share.
+struct TileCounts {
+  unsigned long long next;   // tile to take next
+  unsigned long long list;   // list entries reserved (may exceed the capacity)
+  unsigned long long rest;   // entries whose strings have no planes
+};
+
+// Screens tiles [t_begin, t_end), `batch` at a time per warp.  A warp reserves
+// list entries `chunk` (a multiple of T_FLUSH) at a time; entries past `cap`
+// are counted and not written, and what is left of a warp's last chunk is
+// filled with NO_HIT.  Every warp's lanes take the same branches except in the
+// posting loads.
+__global__ void __launch_bounds__(T_BLOCK) k_screen_tiles(const ProbeView v, const Hit* __restrict__ hits,
+                                                          const Tile* __restrict__ tiles,
+                                                          unsigned long long t_begin, unsigned long long t_end,
+                                                          unsigned batch, unsigned chunk,
+                                                          uint2* __restrict__ list, unsigned long long cap,
+                                                          TileCounts* tc, Counters* ctr) {
+  __shared__ uint2 queues[T_BLOCK / 32][T_CAP];
+  const unsigned lane = threadIdx.x & 31u;
+  uint2* const w = queues[threadIdx.x >> 5];
+  int err = 0;
+  unsigned qn = 0;                     // queued survivors, the same in every lane
+  unsigned long long survivors = 0;
+  unsigned long long at = 0, end = 0;  // the warp's reserved entries
+  auto flush = [&](unsigned from, unsigned n) {  // n <= T_FLUSH entries w[from ..]
+    __syncwarp();
+    if (at == end) {
+      if (lane == 0) at = atomicAdd(&tc->list, (unsigned long long)chunk);
+      at = __shfl_sync(FULL, at, 0);
+      end = at + chunk;
+    }
+#pragma unroll
+    for (unsigned k = 0; k < T_FLUSH; k += 32) {
+      const unsigned long long o = at + k + lane;
+      if (o < cap) list[o] = k + lane < n ? w[from + k + lane] : make_uint2(NO_HIT, 0u);
+    }
+    at += T_FLUSH;
+    survivors += n;
+    __syncwarp();  // the entries were taken before the next write
+  };
+  for (;;) {
+    unsigned long long t0 = 0;
+    if (lane == 0) t0 = t_begin + atomicAdd(&tc->next, (unsigned long long)batch);
+    t0 = __shfl_sync(FULL, t0, 0);
+    if (t0 >= t_end) break;
+    const unsigned long long t1 = min(t_end, t0 + batch);
+    for (unsigned long long t = t0; t < t1; ++t) {
+      const uint4 tile = *reinterpret_cast<const uint4*>(tiles + t);
+      const uint32_t before = (tile.y >> 8) * TILE_POSTS, posts = tile.y & 255u;
+      const int nj = (int)(posts + 31) >> 5;
+      uint32_t sid[TILE_J], L[TILE_J][3], R[TILE_J][3];
+#pragma unroll
+      for (int j = 0; j < TILE_J; ++j) {
+        const uint32_t k = lane + 32u * j;
+        const uint4 rec = *reinterpret_cast<const uint4*>(v.precs + tile.x + min(k, posts - 1));
+        const bool valid = rec.x < v.n_index;
+        if (!valid) err |= 1;
+        sid[j] = k < posts && valid ? rec.x : NO_HIT;
+        L[j][0] = rec.y & SIDE_MASK;
+        L[j][1] = rec.z & SIDE_MASK;
+        L[j][2] = rec.w & SIDE_MASK;
+        R[j][0] = rec.y >> 4 & SIDE_MASK;
+        R[j][1] = rec.z >> 4 & SIDE_MASK;
+        R[j][2] = rec.w >> 4 & SIDE_MASK;
+      }
+      __syncwarp();
+      for (uint32_t k = 0; k < tile.w; ++k) {
+        const uint32_t h = tile.z + k;
+        const uint4 a = reinterpret_cast<const uint4*>(hits + h)[0], b = reinterpret_cast<const uint4*>(hits + h)[1];
+        const uint32_t l0 = b.x & SIDE_MASK, l1 = b.y & SIDE_MASK, l2 = b.z & SIDE_MASK;
+        const uint32_t r0 = b.x >> 4 & SIDE_MASK, r1 = b.y >> 4 & SIDE_MASK, r2 = b.z >> 4 & SIDE_MASK;
+        const unsigned bl = b.w & 0xFFu, br = b.w >> 8 & 0xFFu;
+        // postings of the tile that this hit takes (runs ascend by sid, and a
+        // self join's probe takes those before it)
+        const uint32_t mine = a.z > before ? a.z - before : 0u;
+#pragma unroll
+        for (int j = 0; j < TILE_J; ++j) {
+          if (j < nj) {
+            const unsigned dl = byte_distance(L[j][2], l2, byte_distance(L[j][1], l1, byte_distance(L[j][0], l0, 0)));
+            const unsigned dr = byte_distance(R[j][2], r2, byte_distance(R[j][1], r1, byte_distance(R[j][0], r0, 0)));
+            const bool pass = dl <= bl && dr <= br && lane + 32u * j < mine && sid[j] != NO_HIT;
+            const unsigned m = __ballot_sync(FULL, pass);
+            if (pass) w[qn + __popc(m & lanemask_lt())] = make_uint2(h, sid[j]);
+            qn += __popc(m);
+          }
+        }
+        if (qn >= T_FLUSH) {
+          qn -= T_FLUSH;
+          flush(qn, T_FLUSH);
+        }
+      }
+    }
+  }
+  if (qn) flush(0, qn);
+  for (; at < end; at += T_FLUSH)
+#pragma unroll
+    for (unsigned k = 0; k < T_FLUSH; k += 32)
+      if (at + k + lane < cap) list[at + k + lane] = make_uint2(NO_HIT, 0u);
+  // the host adds the tiles' candidates
+  if (lane == 0 && survivors) atomicAdd(&ctr->filtered, 0ull - survivors);
+  if (err) atomicOr(&ctr->err, (unsigned long long)err);
+}
+
+// Bit-plane verification of the first n list entries.  Entries of strings
+// without planes are counted in tc->rest, the first rest_cap of them also
+// listed in rest.
+template <int MAXW, bool SELF>
+__global__ void __launch_bounds__(T_BLOCK) k_verify_list(const ProbeView v, const Hit* __restrict__ hits,
+                                                         unsigned long long n_hits, const uint2* __restrict__ list,
+                                                         unsigned long long n, uint32_t* __restrict__ rest,
+                                                         unsigned long long rest_cap, TileCounts* tc, AccOut out, Counters* ctr) {
+  __shared__ SecondQueue queues[T_BLOCK / 32];
+  const unsigned lane = threadIdx.x & 31u;
+  SecondQueue& w = queues[threadIdx.x >> 5];
+  unsigned long long cells = 0;
+  int n2 = 0;  // the same in every lane
+  const unsigned long long warp = ((unsigned long long)blockIdx.x * T_BLOCK + threadIdx.x) >> 5;
+  const unsigned long long stride = (unsigned long long)gridDim.x * T_BLOCK;
+  for (unsigned long long base = warp * 32; base < n; base += stride) {
+    const unsigned long long i = base + lane;
+    const uint2 e = i < n ? list[i] : make_uint2(NO_HIT, 0u);
+    bool pass = false;
+    uint32_t q = 0, pi = 0, lim = 0;
+    if (e.x < n_hits && e.y < v.n_index) {  // not NO_HIT
+      const uint4 a = *reinterpret_cast<const uint4*>(hits + e.x);
+      q = a.x;
+      pi = a.w;
+      lim = hits[e.x].lim;
+      if (SELF && q == e.y) {
+        // the probe itself (a colliding run may hold it)
+      } else if (lim >> 16) {
+        const PlaneMatch m = plane_match(v, q, e.y, pi, lim);
+        const int tl = m.i - 1, tr = m.tau + 1 - m.i;
+        const bool right = tr < tl;
+        unsigned c = 0;
+        if (m.li <= SEG_EXACT_MAX || plane_segment(m)) {
+          const int d1 = plane_side<(MAXW - 1) / 2>(m, right, c);
+          pass = d1 <= (right ? tr : tl);
+          lim = (lim & ~0xFFu) | (uint32_t)(d1 & 0xFF);
+        }
+        cells += c;
+      } else {
+        const unsigned long long pos = atomicAdd(&tc->rest, 1ull);
+        if (pos < rest_cap) rest[pos] = (uint32_t)i;
+      }
+    }
+    __syncwarp();
+    const unsigned b = __ballot_sync(FULL, pass);
+    if (pass) {
+      const int slot = n2 + __popc(b & lanemask_lt());
+      w.q[slot] = q;
+      w.sid[slot] = e.y;
+      w.pi[slot] = pi;
+      w.lim[slot] = lim;
+    }
+    n2 += __popc(b);
+    __syncwarp();
+    if (n2 >= 32) verify_second<MAXW, SELF, false>(v, w, n2, out, ctr, cells);
+    __syncwarp();
+  }
+  while (n2) {
+    verify_second<MAXW, SELF, false>(v, w, n2, out, ctr, cells);
+    __syncwarp();
+  }
+  add_counter(&ctr->cells, cells);
+}
+
+// Verification, one thread per entry, of the entries that planes do not
+// serve: all n of the list (rest NULL), the listed ones, or, when more were
+// counted than listed, those of all n whose hit has no lengths.
+template <int MAXW, bool SELF>
+__global__ void __launch_bounds__(T_BLOCK) k_verify_rest(const ProbeView v, const Hit* __restrict__ hits,
+                                                         const uint2* __restrict__ list, unsigned long long n,
+                                                         const uint32_t* __restrict__ rest,
+                                                         unsigned long long rest_cap,
+                                                         const TileCounts* __restrict__ tc, AccOut out, Counters* ctr) {
+  const bool listed = rest && tc->rest <= rest_cap;
+  const unsigned long long m = listed ? tc->rest : n;
+  unsigned long long cells = 0;
+  for (unsigned long long k = (unsigned long long)blockIdx.x * T_BLOCK + threadIdx.x; k < m;
+       k += (unsigned long long)gridDim.x * T_BLOCK) {
+    const uint2 e = list[listed ? (unsigned long long)rest[k] : k];
+    if (e.x == NO_HIT) continue;
+    const uint4 a = *reinterpret_cast<const uint4*>(hits + e.x);
+    if (SELF && a.x == e.y) continue;
+    if (rest && !listed && hits[e.x].lim >> 16) continue;
+    verify_queued_entry<MAXW, SELF, false>(v, a.x, e.y, a.w, out, ctr, cells);
+  }
+  add_counter(&ctr->cells, cells);
 }
 
 // One warp per candidate (long strings): the warp walks candidates
@@ -1090,7 +1480,7 @@ __global__ void __launch_bounds__(FB) k_fused_self(const ProbeView v, int ppi, i
           if (lanes.thread_rank() == 0) hv = atomicAdd(&work[2], (unsigned long long)lanes.size());
           hv = lanes.shfl(hv, 0) + lanes.thread_rank();
           if (hv < heavy_cap) {
-            heavy[hv] = Hit{q, b, cnt, 0u, 0ull, 0ull};
+            heavy[hv] = Hit{q, b, cnt, 0u, {{0u, 0u, 0u}}, 0u};
             n_cand += cnt;
             return;
           }
@@ -1361,7 +1751,8 @@ static void launch_verify(const Ctx& c, const ProbeView& v, const Hit* hits, con
                                         (c_end - c_begin + (unsigned long long)Q_BLOCK * S_RUN - 1) /
                                             ((unsigned long long)Q_BLOCK * S_RUN), Q_BLOCK);
     k_verify_queued<MAXW, SELF, MULTI><<<gq, Q_BLOCK, 0, c.stream>>>(v, hits, off, n_hits, c_begin, c_end, out, ctr,
-                                                                    nullptr, queued_chunk(c_end - c_begin, gq));
+                                                                    nullptr,
+                                                                    queued_chunk(c_end - c_begin, gq * Q_WARPS));
     PJ_LAUNCHED("k_verify_queued");
     return;
   }
@@ -1372,6 +1763,64 @@ static void launch_verify(const Ctx& c, const ProbeView& v, const Hit* hits, con
   k_verify_hits<MAXW, SELF, MULTI><<<grid, block, 0, c.stream>>>(v, hits, off, n_hits, c_begin, c_end, out, ctr,
                                                                   nullptr);
   PJ_LAUNCHED("k_verify_hits");
+}
+
+// Hits from which a chunk is grouped by run and verified tile by tile
+// (PJ_TILES_MIN_HITS overrides).
+constexpr unsigned long long TILES_MIN_HITS = 1ull << 16;
+
+// The hits of a chunk grouped by posting run, and the tiles over them.
+struct HitTiles {
+  DBuf<Hit> hits;
+  DBuf<Tile> tiles;
+  DBuf<unsigned long long> totals;  // candidates, tiles, tiles written
+  unsigned long long n_tiles = 0;   // 0: not grouped
+  // one tile range's survivors
+  DBuf<uint2> list;
+  DBuf<uint32_t> rest;
+  DBuf<TileCounts> counts;
+};
+
+// List entries of one tile range (2 GiB), and listed entries without planes.
+constexpr unsigned long long LIST_MAX = 1ull << 28;
+constexpr unsigned long long REST_MAX = 1ull << 20;
+
+// Screens tiles [t_begin, t_end); returns the list entries taken (more than
+// the list holds: the range has to be screened again in smaller parts).
+static unsigned long long screen_tiles(const Ctx& c, const ProbeView& v, HitTiles& t, unsigned long long t_begin,
+                                       unsigned long long t_end, Counters* ctr) {
+  const unsigned long long n = t_end - t_begin;
+  const unsigned grid = persistent_grid(k_screen_tiles, (n + T_BLOCK / 32 - 1) / (T_BLOCK / 32), T_BLOCK);
+  const unsigned long long warps = (unsigned long long)grid * (T_BLOCK / 32);
+  const unsigned batch = (unsigned)std::min<unsigned long long>(16, std::max<unsigned long long>(1, n / (warps * 16)));
+  // at most 1/8 of the list in the warps' unfinished chunks
+  const unsigned chunk = t.list.n >= warps * 8 * 4 * T_FLUSH ? 4 * T_FLUSH : T_FLUSH;
+  PJ_CUDA(cudaMemsetAsync(t.counts.p, 0, sizeof(TileCounts), c.stream));
+  k_screen_tiles<<<grid, T_BLOCK, 0, c.stream>>>(v, t.hits.p, t.tiles.p, t_begin, t_end, batch, chunk, t.list.p,
+                                                 t.list.n, t.counts.p, ctr);
+  PJ_LAUNCHED("k_screen_tiles");
+  TileCounts h{};
+  PJ_CUDA(cudaMemcpyAsync(&h, t.counts.p, sizeof(h), cudaMemcpyDeviceToHost, c.stream));
+  c.sync();
+  return h.list;
+}
+
+// Verifies the first n entries of t's list.
+template <int MAXW, bool SELF>
+static void launch_list(const Ctx& c, const ProbeView& v, const HitTiles& t, unsigned long long n, AccOut out,
+                        Counters* ctr) {
+  if (MAXW <= 5 && v.pplanes) {
+    const unsigned g = persistent_grid(k_verify_list<MAXW <= 5 ? MAXW : 5, SELF>, (n + T_BLOCK - 1) / T_BLOCK, T_BLOCK);
+    k_verify_list<MAXW <= 5 ? MAXW : 5, SELF><<<g, T_BLOCK, 0, c.stream>>>(v, t.hits.p, t.hits.n, t.list.p, n, t.rest.p, t.rest.n,
+                                                                          t.counts.p, out, ctr);
+    PJ_LAUNCHED("k_verify_list");
+  }
+  const bool all = !(MAXW <= 5 && v.pplanes);
+  const unsigned gr = persistent_grid(k_verify_rest<MAXW, SELF>,
+                                      ((all ? n : t.rest.n) + T_BLOCK - 1) / T_BLOCK, T_BLOCK);
+  k_verify_rest<MAXW, SELF><<<gr, T_BLOCK, 0, c.stream>>>(v, t.hits.p, t.list.p, n, all ? nullptr : t.rest.p,
+                                                          t.rest.n, t.counts.p, out, ctr);
+  PJ_LAUNCHED("k_verify_rest");
 }
 
 template <bool SELF, bool MULTI>
@@ -1482,6 +1931,7 @@ static void pinned_put(void* p, size_t bytes) {
 //   PJ_LAUNCH_CANDS      candidates per verification launch (default 1 Gi)
 //   PJ_ACCEPT_INITIAL    initial accepted-match capacity  (default 4 Mi)
 //   PJ_GRAPH_MAX_GROUPS  groups of a recorded self join   (default 256 Mi)
+//   PJ_TILES_MIN_HITS    hits grouped by run              (default 64 Ki)
 //   PJ_GRAPH_TIGHT       1: record self joins with half their counts as
 //                        capacities, so that every replay overflows
 static unsigned long long env_knob(const char* name, unsigned long long dflt) {
@@ -1555,6 +2005,37 @@ struct AcceptBuf {
   }
 };
 
+// Groups n hits over the postings [0, n_postings) of v's index; returns the
+// number of candidates.
+static unsigned long long group_hits(const Ctx& c, const ProbeView& v, DBuf<Hit>& hits, unsigned long long n,
+                                     HitTiles& t) {
+  const unsigned long long np = v.n_postings;
+  DBuf<uint32_t> cnt(c, 2 * np), off(c, np), rank(c, n);
+  uint32_t* longest = cnt.p + np;
+  t.totals.reset(c, 3);
+  PJ_CUDA(cudaMemsetAsync(cnt.p, 0, cnt.bytes(), c.stream));
+  PJ_CUDA(cudaMemsetAsync(t.totals.p, 0, t.totals.bytes(), c.stream));
+  const unsigned gh = (unsigned)std::min<unsigned long long>((n + BLOCK - 1) / BLOCK, sm_grid_cap(8));
+  const unsigned gp = (unsigned)std::min<unsigned long long>((np + BLOCK - 1) / BLOCK, sm_grid_cap(8));
+  k_run_count<<<gh, BLOCK, 0, c.stream>>>(hits.p, n, cnt.p, longest, rank.p, t.totals.p);
+  PJ_LAUNCHED("k_run_count");
+  k_tile_count<<<gp, BLOCK, 0, c.stream>>>(cnt.p, longest, np, t.totals.p);
+  PJ_LAUNCHED("k_tile_count");
+  exclusive_scan<uint32_t>(c, cnt.p, off.p, np);
+  t.hits.reset(c, n);
+  k_run_scatter<<<gh, BLOCK, 0, c.stream>>>(hits.p, n, off.p, rank.p, t.hits.p);
+  PJ_LAUNCHED("k_run_scatter");
+  unsigned long long h[2] = {0, 0};
+  PJ_CUDA(cudaMemcpyAsync(h, t.totals.p, sizeof(h), cudaMemcpyDeviceToHost, c.stream));
+  c.sync();
+  t.n_tiles = h[1];
+  t.tiles.reset(c, t.n_tiles);
+  k_tile_emit<<<gp, BLOCK, 0, c.stream>>>(cnt.p, longest, off.p, np, t.tiles.p, t.n_tiles, t.totals.p);
+  PJ_LAUNCHED("k_tile_emit");
+  hits.release();
+  return h[0];
+}
+
 // Probe + verify for all probing strings, in chunks of probing strings whose
 // groups fit the hit buffer; then the short-string fallback.  Returns the
 // number of accepted matches (the buffer holds min(that, out.cap)).
@@ -1563,7 +2044,9 @@ struct AcceptBuf {
 template <bool SELF, bool MULTI>
 static void probe_chunk(const Ctx& c, const ProbeView& v, unsigned long long n_groups, Counters* ctr,
                         DBuf<uint32_t>& gcount, DBuf<uint32_t>& goff, DBuf<Hit>& hits, DBuf<unsigned long long>& cnt,
-                        DBuf<unsigned long long>& off, unsigned long long& n_hits, unsigned long long& n_cand) {
+                        DBuf<unsigned long long>& off, unsigned long long& n_hits, unsigned long long& n_cand,
+                        HitTiles* tiles = nullptr) {
+  if (tiles) tiles->n_tiles = 0;
   gcount.reset(c, n_groups);
   goff.reset(c, n_groups);
   DBuf<unsigned long long> gmask(c, n_groups);
@@ -1584,6 +2067,11 @@ static void probe_chunk(const Ctx& c, const ProbeView& v, unsigned long long n_g
                                                         n_hits);
   PJ_LAUNCHED("k_group_hits");
   trace_mark(c, "join: probe (hits)");
+  if (tiles && n_hits >= env_knob("PJ_TILES_MIN_HITS", TILES_MIN_HITS)) {
+    n_cand = group_hits(c, v, hits, n_hits, *tiles);
+    trace_mark(c, "join: group hits by run");
+    return;
+  }
   cnt.reset(c, n_hits + 1);
   off.reset(c, n_hits + 1);
   PJ_CUDA(cudaMemsetAsync(cnt.p + n_hits, 0, sizeof(unsigned long long), c.stream));
@@ -1861,7 +2349,13 @@ static void probe_and_verify(const Ctx& c, const ProbeView& v0, uint32_t fb_coun
   DBuf<Hit> hits;
   DBuf<uint32_t> gcount, goff;
   DBuf<unsigned long long> cnt, off;
-  unsigned long long total_cand = 0, verified = 0;
+  HitTiles tiles;
+  // run-major verification: extension mode with the side screen, no warp-per-
+  // candidate range, no device budget (grouping keeps a second copy of the
+  // hits)
+  const bool use_tiles = !MULTI && !v0.pair_mode && v0.queued && v0.hit_sides && !c.budget &&
+                         (uint64_t)v0.warp_q_cut >= (uint64_t)v0.pbegin + v0.pcount;
+  unsigned long long total_cand = 0, verified = 0, tile_cand = 0;
   bool fused_done = false;
   ProbeView vc = v0;  // the probes of the chunked pipeline
   if (SELF && !MULTI && v0.fused && v0.pcount) {  // the fused persistent kernel over the probes from fused_q_cut
@@ -1891,7 +2385,8 @@ static void probe_and_verify(const Ctx& c, const ProbeView& v0, uint32_t fb_coun
     }
     tp.start();
     unsigned long long n_hits = 0, n_cand = 0;
-    probe_chunk<SELF, MULTI>(c, v, n_groups, ctr, gcount, goff, hits, cnt, off, n_hits, n_cand);
+    probe_chunk<SELF, MULTI>(c, v, n_groups, ctr, gcount, goff, hits, cnt, off, n_hits, n_cand,
+                             use_tiles ? &tiles : nullptr);
     if (n_hits == 0) {
       tp.stop();
       tm.probe += tp.ms();
@@ -1900,8 +2395,10 @@ static void probe_and_verify(const Ctx& c, const ProbeView& v0, uint32_t fb_coun
     }
     tp.stop();
     tm.probe += tp.ms();
-    debug_dump(c, "hits", hits.p, n_hits * sizeof(Hit));
-    debug_dump(c, "cand_off", off.p, (n_hits + 1) * sizeof(unsigned long long));
+    if (!tiles.n_tiles) {
+      debug_dump(c, "hits", hits.p, n_hits * sizeof(Hit));
+      debug_dump(c, "cand_off", off.p, (n_hits + 1) * sizeof(unsigned long long));
+    }
     h.candidates += n_cand;
     h.hits += n_hits;
     total_cand += n_cand;
@@ -1913,6 +2410,58 @@ static void probe_and_verify(const Ctx& c, const ProbeView& v0, uint32_t fb_coun
       tm.verify += tv.ms();
       verified += n_cand;
       trace_mark(c, "join: verify (distinct pairs)");
+      done += v.pcount;
+      continue;
+    }
+    if (tiles.n_tiles) {
+      // The list holds a quarter of the candidates (about 9% survive on short
+      // strings at tau = 4), at most LIST_MAX; a range whose survivors do not
+      // fit is screened again in halves.  Accepted matches never exceed the
+      // list, so the verification never runs twice.
+      const unsigned long long T = tiles.n_tiles;
+      const unsigned long long want =
+          std::min({n_cand + (1ull << 20), std::max(n_cand / 4, 1ull << 22), LIST_MAX, env_knob("PJ_LAUNCH_CANDS", LIST_MAX)});
+      if (tiles.list.n < want) tiles.list.reset(c, want);
+      if (!tiles.rest.p) tiles.rest.reset(c, REST_MAX);
+      if (!tiles.counts.p) tiles.counts.reset(c, 1);
+      tv.start();
+      double share = (double)tiles.list.n / (0.2 * (double)n_cand);  // of the tiles whose survivors fit, expected
+      for (unsigned long long tb = 0; tb < T;) {
+        const unsigned long long step =
+            std::max<unsigned long long>(1, (unsigned long long)(std::min(1.0, share) * (double)T));
+        const unsigned long long te = std::min(T, tb + step);
+        Counters saved{};
+        PJ_CUDA(cudaMemcpyAsync(&saved, ctr, sizeof(saved), cudaMemcpyDeviceToHost, c.stream));
+        const unsigned long long n = screen_tiles(c, v, tiles, tb, te, ctr);
+        if (n > tiles.list.n) {
+          PJ_CUDA(cudaMemcpyAsync(ctr, &saved, sizeof(saved), cudaMemcpyHostToDevice, c.stream));
+          c.sync();
+          if (step == 1) {  // one tile's survivors (at most TILE_POSTS * TILE_HITS and a chunk)
+            tiles.list.reset(c, (unsigned long long)TILE_POSTS * TILE_HITS + 8 * T_FLUSH);
+          } else {
+            share = 0.5 * (double)step / (double)T;
+          }
+          continue;
+        }
+        share = std::min(2.0 * (double)step / (double)T, 0.9 * (double)tiles.list.n / (double)std::max(1ull, n) *
+                                                             ((double)(te - tb) / (double)T));
+        if (n) {
+          if (acc.last + n > acc.cap) acc.reserve(std::max(acc.last + n, acc.cap + acc.cap / 2));
+          acc.run(
+              [&](AccOut o) {
+#define PJ_CALL(W) launch_list<W, SELF>(c, v, tiles, n, o, ctr)
+                PJ_BY_TAU(v.tau, PJ_CALL);
+#undef PJ_CALL
+              },
+              [&](unsigned long long after) { return 2 * after; });
+        }
+        tb = te;
+      }
+      tv.stop();
+      tm.verify += tv.ms();
+      verified += n_cand;
+      tile_cand += n_cand;
+      trace_mark(c, "join: verify (tiles)");
       done += v.pcount;
       continue;
     }
@@ -1991,6 +2540,7 @@ static void probe_and_verify(const Ctx& c, const ProbeView& v0, uint32_t fb_coun
   c.sync();
   // the chunked pipeline counts candidates and hits on the host, the fused
   // kernel its candidates on the device
+  h.filtered += tile_cand;  // the tiles took their survivors off
   h.candidates = cand + (fused_done ? h.candidates : 0ull);
   h.hits = nh;
   if (h.err)
@@ -2495,6 +3045,7 @@ static ProbeView index_side(const pj_index& idx, const Partition& part) {
   v.table_pb = part.presence_bytes;
   v.precs = part.precs.p;
   v.ibm = idx.sbm.p;
+  v.iplanes = idx.splanes.p;
   v.mask = part.table.n - 1;
   v.postings = part.postings.p;
   v.n_postings = part.n_records;
@@ -2705,7 +3256,7 @@ static void record_self_plan(const Ctx& c, const ProbeView& v, SelfPlan& P) {
   do {                                                                                                         \
     const unsigned gv = persistent_grid(k_verify_queued<W, true, false>, ~0ull >> 8, Q_BLOCK);                  \
     k_verify_queued<W, true, false><<<gv, Q_BLOCK, 0, c.stream>>>(v, P.hits.p, P.hoff.p, P.cap_hits, 0, 0, acc,  \
-                                                                  ctr, &sz->hits, queued_chunk(P.n_cand, gv));  \
+                                                                  ctr, &sz->hits, 0);  \
     PJ_LAUNCHED("k_verify_queued");                                                                            \
   } while (0)
     PJ_BY_TAU(v.tau, PJ_CALL);
@@ -3001,6 +3552,8 @@ static void self_join_impl(pj_index& idx, int tau, pj_result* out, bool on_devic
   v.pid = idx.perm.p;
   v.pref = idx.sref.p;
   v.pbm = idx.sbm.p;
+  v.pplanes = idx.splanes.p;
+  v.nplanes = planes_used(idx.byte_bits, true);
   v.phash = idx.sph.p;
   v.key_shift = bits_for(idx.n);
   v.gorder = part.gorder[1].p;
@@ -3086,6 +3639,8 @@ static void probe_join_impl(const Ctx& c, const pj_index& idx, const Partition& 
   v.pcount = R.n;
   v.pid = nullptr;
   v.pbm = R.bm.p;
+  v.pplanes = R.planes.p;
+  v.nplanes = planes_used(idx.byte_bits, false);
   v.key_shift = bits_for(idx.n);
   v.gorder = part.gorder[0].p;
   TuneResult mode;
@@ -3141,6 +3696,8 @@ void query_multi_impl(const Ctx& c, pj_index& idx, const ProbeSet& R, const uint
   v.pcount = R.n;
   v.pid = nullptr;
   v.pbm = R.bm.p;
+  v.pplanes = R.planes.p;
+  v.nplanes = planes_used(idx.byte_bits, false);
   v.key_shift = bits_for(idx.n);
   v.ptau = d_tau.p;
   v.qgoff = d_qgoff.p;
@@ -3162,13 +3719,14 @@ static_assert(sizeof(Counters) == 64, "plan counters are 64 bytes");
 // group offsets of every q >= n equal the total (group_of searches all cap_q).
 __global__ void k_plan_groups(const uint8_t* __restrict__ bytes, const uint64_t* __restrict__ off,
                               const uint8_t* __restrict__ tau, uint32_t cap_q, const PlanSizes* __restrict__ sizes,
-                              uint32_t* __restrict__ len, Sig* __restrict__ bm,
-                              unsigned long long* __restrict__ gcnt) {
+                              uint32_t* __restrict__ len, Sig* __restrict__ bm, Planes* __restrict__ planes,
+                              ByteBits bb, unsigned long long* __restrict__ gcnt) {
   const unsigned long long n = sizes->n;
   for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < cap_q; q += gridDim.x * blockDim.x) {
     if (q < n) {
       len[q] = (uint32_t)(off[q + 1] - off[q]);
       bm[q] = char_signature(bytes + off[q], (int)len[q]);
+      if (planes) planes[q] = string_planes(bytes + off[q], (int)len[q], bb);
       gcnt[q] = (unsigned long long)groups_per_probe((int)tau[q], false);
     } else {
       gcnt[q] = 0;
@@ -3207,6 +3765,8 @@ void record_query_plan(const Ctx& c, const pj_index& idx, const PlanDev& d) {
   v.qgoff = d.qgoff;
   v.parts = d.parts;
   v.pbm = d.bm;
+  v.pplanes = d.planes;
+  v.nplanes = planes_used(idx.byte_bits, false);
   bool has_short = false;
   for (int t = 0; t <= tau_max; ++t) has_short |= idx.parts[t].first > 0;
   Counters* ctr = static_cast<Counters*>(d.counters);
@@ -3214,7 +3774,8 @@ void record_query_plan(const Ctx& c, const pj_index& idx, const PlanDev& d) {
   PJ_CUDA(cudaMemsetAsync(ctr, 0, sizeof(Counters), c.stream));
 
   // A4: groups of every query, lookups, hits, candidate offsets
-  k_plan_groups<<<stride_grid(d.cap_q), 256, 0, c.stream>>>(d.bytes, d.off, d.tau, d.cap_q, sz, d.len, d.bm, d.gcnt);
+  k_plan_groups<<<stride_grid(d.cap_q), 256, 0, c.stream>>>(d.bytes, d.off, d.tau, d.cap_q, sz, d.len, d.bm, d.planes,
+                                                        idx.byte_bits, d.gcnt);
   PJ_LAUNCHED("k_plan_groups");
   exclusive_scan_dn<unsigned long long>(c, d.gcnt, d.qgoff, d.cap_q, nullptr, &sz->groups);
   const unsigned g1 = persistent_grid(k_group_counts<false, true>, (d.cap_groups + BLOCK - 1) / BLOCK);
@@ -3235,7 +3796,7 @@ void record_query_plan(const Ctx& c, const pj_index& idx, const PlanDev& d) {
   do {                                                                                                         \
     const unsigned gv = persistent_grid(k_verify_queued<W, false, true>, ~0ull >> 8, Q_BLOCK);                  \
     k_verify_queued<W, false, true><<<gv, Q_BLOCK, 0, c.stream>>>(v, d.hits, d.hoff, d.cap_hits, 0, 0, acc, ctr, \
-                                                                  &sz->hits, Q_CHUNK);                         \
+                                                                  &sz->hits, 0);                         \
     PJ_LAUNCHED("k_verify_queued");                                                                            \
     if (has_short) {                                                                                           \
       const unsigned gf = persistent_grid(k_fallback<W, false, true>, (d.cap_q + BLOCK - 1) / BLOCK);           \
@@ -3349,7 +3910,7 @@ int pj_join(const pj_strings* R, const pj_strings* S, int tau, const pj_options*
     pj::build_partition(*tmp, tau, tmp->parts[tau]);
     {  // the probe set's buffers refer to tmp->ctx: released before tmp
       pj::ProbeSet P;
-      pj::upload_probe_set(tmp->ctx, *R, P);
+      pj::upload_probe_set(tmp->ctx, *tmp, *R, P);
       pj::probe_join_impl(tmp->ctx, *tmp, tmp->parts[tau], P, out, tmp->results_on_device);
       tmp->ctx.sync();
     }
@@ -3378,7 +3939,7 @@ int pj_query(pj_index* idx, const pj_strings* batch, int tau, pj_result* out) {
     float part_ms = 0.f;
     pj::Partition& part = pj::ensure_partition(*idx, tau, &part_ms);
     pj::ProbeSet P;
-    pj::upload_probe_set(idx->ctx, *batch, P);
+    pj::upload_probe_set(idx->ctx, *idx, *batch, P);
     pj::probe_join_impl(idx->ctx, *idx, part, P, out, idx->results_on_device);
     out->stats.partition_ms = part_ms;
     return PJ_OK;
@@ -3406,7 +3967,7 @@ int pj_query_multi(pj_index* idx, const pj_strings* batch, const uint8_t* taus, 
     for (int t = 0; t < (int)idx->parts.size(); ++t)
       if (seen[t]) pj::ensure_partition(*idx, t, nullptr);
     pj::ProbeSet P;
-    pj::upload_probe_set(idx->ctx, *batch, P);
+    pj::upload_probe_set(idx->ctx, *idx, *batch, P);
     pj::query_multi_impl(idx->ctx, *idx, P, taus, out, idx->results_on_device);
     return PJ_OK;
   } catch (const pj::Error& e) {

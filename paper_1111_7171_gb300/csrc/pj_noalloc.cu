@@ -195,7 +195,7 @@ void query_noalloc(pj_index& idx, const pj_strings& batch, int tau, pj_pair* out
   c.alloc_ctx = &bump;
 
   ProbeSet R;
-  upload_probe_set(c, batch, R);  // device input: lengths only, in the scratch
+  upload_probe_set(c, idx, batch, R, false);  // device input: lengths and signatures only, in the scratch
   DBuf<NaCounters> ctr(c, 1);
   PJ_CUDA(cudaMemsetAsync(ctr.p, 0, sizeof(NaCounters), c.stream));
 

@@ -37,6 +37,7 @@ struct pj_plan {
   pj::DBuf<uint32_t> len, gcounts, goff, flags, pos, acc_ed0, acc_ed1;
   pj::DBuf<unsigned long long> gcnt, qgoff, gmask, hcnt, hoff, acc_key0, acc_key1;
   pj::DBuf<pj::Sig> bm;
+  pj::DBuf<pj::Planes> planes;
   pj::DBuf<pj::PartView> parts;
   pj::DBuf<unsigned char> counters, arena;
   pj::DBuf<pj::Hit> hits;
@@ -50,7 +51,7 @@ struct pj_plan {
   uint64_t device_bytes() const {
     return bytes.bytes() + tau.bytes() + off.bytes() + sizes.bytes() + len.bytes() + gcounts.bytes() + goff.bytes() +
            flags.bytes() + pos.bytes() + acc_ed0.bytes() + acc_ed1.bytes() + gcnt.bytes() + qgoff.bytes() +
-           gmask.bytes() + bm.bytes() + hcnt.bytes() + hoff.bytes() + acc_key0.bytes() + acc_key1.bytes() + parts.bytes() + counters.bytes() +
+           gmask.bytes() + bm.bytes() + planes.bytes() + hcnt.bytes() + hoff.bytes() + acc_key0.bytes() + acc_key1.bytes() + parts.bytes() + counters.bytes() +
            arena.bytes() + hits.bytes();
   }
   uint64_t host_bytes() const {
@@ -74,6 +75,7 @@ struct pj_plan {
     pj::DBuf<unsigned long long>* b64[] = {&gcnt, &qgoff, &gmask, &hcnt, &hoff, &acc_key0, &acc_key1};
     for (auto* b : b64) b->release();
     bm.release();
+    planes.release();
     parts.release();
     counters.release();
     arena.release();
@@ -234,6 +236,7 @@ void create(pj_plan& P, pj_index& idx, const pj_plan_options& o) {
   P.sizes.reset(P.ctx, 1);
   P.len.reset(P.ctx, d.cap_q);
   P.bm.reset(P.ctx, d.cap_q);
+  if (idx.splanes.p) P.planes.reset(P.ctx, d.cap_q);
   P.gcnt.reset(P.ctx, d.cap_q);
   P.qgoff.reset(P.ctx, d.cap_q);
   P.gcounts.reset(P.ctx, d.cap_groups);
@@ -246,6 +249,7 @@ void create(pj_plan& P, pj_index& idx, const pj_plan_options& o) {
   d.sizes = P.sizes.p;
   d.len = P.len.p;
   d.bm = P.bm.p;
+  d.planes = P.planes.p;
   d.gcnt = P.gcnt.p;
   d.qgoff = P.qgoff.p;
   d.gcounts = P.gcounts.p;

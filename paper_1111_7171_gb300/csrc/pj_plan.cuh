@@ -42,6 +42,7 @@ struct PlanDev {
   // pipeline state
   uint32_t* len;                  // cap_q
   Sig* bm;                        // cap_q character signatures
+  Planes* planes;                 // cap_q bit planes (NULL: the index has none)
   unsigned long long* gcnt;       // cap_q groups per query
   unsigned long long* qgoff;      // cap_q group offsets
   const PartView* parts;          // tau_max + 1 thresholds

@@ -15,17 +15,29 @@
 namespace pj {
 
 // A lookup with a non-empty posting run.  pi = p | (i << 16) | (tau << 24);
-// the tau byte is used by multi-threshold batches only.  sl and sr are the
-// side signatures (side_signature) of the probe left of the selected
-// substring, s[0, p), and right of it, s[p + l_i, |s|), for the screen in
-// front of extension verification.
+// the tau byte is used by multi-threshold batches only.  sides holds the
+// probe's side signatures left and right of the selected substring, s[0, p)
+// and s[p + l_i, |s|), for the screen in front of extension verification;
+// lim = left limit | right limit << 8 | l << 16 | |s| << 24: the largest
+// count differences (side_distances) that the sides' thresholds and length
+// differences leave, and the two lengths when both are at most PLANE_LEN
+// (else 0).
 struct __align__(16) Hit {
   uint32_t q;
   uint32_t begin;
   uint32_t count;
   uint32_t pi;
-  unsigned long long sl, sr;
+  SidePair sides;
+  uint32_t lim;
 };
+
+__host__ __device__ __forceinline__ uint32_t hit_limits(int tau, int i, int ls, int l, int p, int P, int li) {
+  const int dl = p > P ? p - P : P - p;
+  const int dr0 = (ls - p) - (l - P), dr = dr0 < 0 ? -dr0 : dr0;
+  const uint32_t lo = (uint32_t)max(0, 2 * (i - 1) - dl), hi = (uint32_t)max(0, 2 * (tau + 1 - i) - dr);
+  const uint32_t lens = l <= PLANE_LEN && ls <= PLANE_LEN ? (uint32_t)l << 16 | (uint32_t)ls << 24 : 0u;
+  return lo | hi << 8 | lens;
+}
 
 // One threshold's segment index, as seen by the kernels.
 struct PartView {
@@ -86,8 +98,13 @@ struct ProbeView {
   // character-count bound)
   const Sig* pbm;
   const Sig* ibm;
+  // bit planes of the probing and the indexed strings (NULL: none) and how
+  // many are in use
+  const Planes* pplanes;
+  const Planes* iplanes;
+  int nplanes;
   int queued;     // thread-per-candidate verification with a screen and per-warp queues
-  int hit_sides;  // hits carry the probe's side signatures (Hit::sl, sr) and the queued screen tests them
+  int hit_sides;  // hits carry the probe's side signatures and the queued screen tests them
   int pair_mode;  // 1: mode L (distinct candidate pairs verified once over the whole strings)
   int pair_warp;  // mode L: one warp per pair instead of one thread
   int share_prefix;  // mode L: consecutive pairs of a probe share the DP rows of common prefixes (Sec. 5.3)
@@ -274,6 +291,15 @@ __host__ __device__ __forceinline__ HitCtx hit_ctx(const ProbeView& v, const Hit
   return c;
 }
 
+// The reported pair key of probe q and indexed sid r.
+__host__ __device__ __forceinline__ unsigned long long match_key(const ProbeView& v, bool self, uint32_t q, uint32_t r) {
+  const uint32_t qid = v.pid ? v.pid[q] : q;
+  const uint32_t rid = v.iperm[r];
+  const uint32_t ka = self ? min(qid, rid) : qid;
+  const uint32_t kb = self ? max(qid, rid) : rid;
+  return ((unsigned long long)ka << v.key_shift) | kb;
+}
+
 // Extension verification (Sec. 5.2, Alg. 3) of indexed string r against the
 // hit described by hc, r already screened (a valid sid, not the probe
 // itself).  Returns true with the pair key and ed = d_l + d_r when accepted.
@@ -303,15 +329,40 @@ __host__ __device__ __forceinline__ bool verify_screened(const ProbeView& v, boo
     // segment match; hashed ones are compared
     if (hc.p + li <= hc.ls && verify_ext<MAXW>(hc.s, hc.ls, rb, lr, i, hc.p, li, P, v.tau,
                                                li > SEG_EXACT_MAX, ed, cells)) {
-      const uint32_t qid = v.pid ? v.pid[hc.q] : hc.q;
-      const uint32_t rid = v.iperm[r];
-      const uint32_t ka = self ? min(qid, rid) : qid;
-      const uint32_t kb = self ? max(qid, rid) : rid;
-      key = ((unsigned long long)ka << v.key_shift) | kb;
+      key = match_key(v, self, hc.q, r);
       ok = true;
     }
   }
   return ok;
+}
+
+// The match of probe q and indexed sid r described by pi and lim (lengths not
+// 0), with both strings' planes.
+__host__ __device__ __forceinline__ PlaneMatch plane_match(const ProbeView& v, uint32_t q, uint32_t r, uint32_t pi,
+                                                           uint32_t lim) {
+  PlaneMatch m;
+#ifdef __CUDA_ARCH__
+  const uint4* x = reinterpret_cast<const uint4*>(v.pplanes + q);
+  const uint4* y = reinterpret_cast<const uint4*>(v.iplanes + r);
+  const uint4 x0 = x[0], x1 = x[1], y0 = y[0], y1 = y[1];
+  m.X[0] = x0.x; m.X[1] = x0.y; m.X[2] = x0.z; m.X[3] = x0.w;
+  m.X[4] = x1.x; m.X[5] = x1.y; m.X[6] = x1.z; m.X[7] = x1.w;
+  m.Y[0] = y0.x; m.Y[1] = y0.y; m.Y[2] = y0.z; m.Y[3] = y0.w;
+  m.Y[4] = y1.x; m.Y[5] = y1.y; m.Y[6] = y1.z; m.Y[7] = y1.w;
+#else
+  for (int b = 0; b < 8; ++b) {
+    m.X[b] = v.pplanes[q].w[b];
+    m.Y[b] = v.iplanes[r].w[b];
+  }
+#endif
+  m.tau = v.tau;
+  m.p = (int)(pi & 0xFFFFu);
+  m.i = (int)(pi >> 16 & 0xFFu);
+  m.lr = (int)(lim >> 16 & 0xFFu);
+  m.ls = (int)(lim >> 24);
+  m.wide = v.nplanes > 6;
+  segment_m(m.lr, v.tau + 1, v.seg_magic, v.scheme, m.i, m.P, m.li);
+  return m;
 }
 
 // The screen in front of every verification: r must be a valid sid (else

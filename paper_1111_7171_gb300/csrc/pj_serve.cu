@@ -95,7 +95,7 @@ void run_batch(pj_server& S, const Ctx& c, pj_plan* plan, std::vector<std::share
       if (code != PJ_OK) msg = pj_last_error();
     } else {  // no plan, or one request larger than the plan's limits
       ProbeSet P;
-      upload_probe_set(c, in, P);
+      upload_probe_set(c, *S.idx, in, P);
       query_multi_impl(c, *S.idx, P, taus.data(), &res, false);
     }
   } catch (const Error& e) {

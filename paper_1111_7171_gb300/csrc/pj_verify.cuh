@@ -12,6 +12,10 @@
 
 namespace pj {
 
+// Longest string that has bit planes: a side's cells (up to one bit more
+// than its length and the threshold 4) fit 32 bits.
+constexpr int PLANE_LEN = 28;
+
 #ifndef __CUDA_ARCH__
 using std::abs;
 using std::max;
@@ -522,6 +526,116 @@ __device__ __forceinline__ bool verify_ext_warp(const uint8_t* s, int ls, const 
   return ok;
 }
 #endif
+
+// VERIFYSTRINGPAIR of two sides in bit planes (Planes): min(T + 1, ED(x, y))
+// for sides of nx, ny characters that start at bit sx of X's planes and bit sy
+// of Y's; nx + T <= 31.
+//
+// Furthest-reaching form of the banded DP of Sec. 5.1: on each diagonal d = j
+// - i of the length-aware band only the furthest cell reached with e edits
+// matters, and a diagonal's matches are free.  A cell is one bit, 1 << i, so
+// the furthest of several is their maximum.  E[k] has bit i set where x[i] ==
+// y[i + d_k]: one xor per plane for all i at once.  Adding the cell's bit to
+// E[k] carries it over the matches that start at i, and the bit it lands on,
+// the first one not in E[k], is the cell that the matches lead to (a cell
+// that starts no match stays; bits of E[k] elsewhere are masked off).  A
+// substitution or deletion moves one bit up, to its own diagonal or the one
+// below, an insertion to the diagonal above without moving.  Cells past an end
+// of the matrix cost one edit more than the cell at the end and reach the
+// result's diagonal no earlier.  The pair's distance is the first e whose cell
+// on diagonal D = ny - nx reaches bit nx.  cells counts the cells evaluated (T
+// + 1 per e).
+template <int T>
+__host__ __device__ __forceinline__ int plane_distance(const uint32_t (&X)[8], int sx, int nx, const uint32_t (&Y)[8],
+                                                       int sy, int ny, bool wide, unsigned& cells) {
+  constexpr int W = T + 1;
+  const int D = ny - nx;
+  int res = T + 1;
+  if (D <= T && D >= -T) {
+    const int up = (T - D) >> 1;  // diagonals d_k = k - up, k = 0 .. T
+    uint32_t M[W];
+#pragma unroll
+    for (int k = 0; k < W; ++k) M[k] = 0;
+#pragma unroll
+    for (int b = 0; b < 6; ++b) {
+      const uint32_t x = X[b] >> sx, y = (Y[b] >> sy) << up;
+#pragma unroll
+      for (int k = 0; k < W; ++k) M[k] |= x ^ (y >> k);
+    }
+    if (wide) {
+#pragma unroll
+      for (int b = 6; b < 8; ++b) {
+        const uint32_t x = X[b] >> sx, y = (Y[b] >> sy) << up;
+#pragma unroll
+        for (int k = 0; k < W; ++k) M[k] |= x ^ (y >> k);
+      }
+    }
+    const uint32_t vx = (1u << nx) - 1u, vy = ((1u << ny) - 1u) << up, goal = 1u << nx;
+    const int kres = D + up;
+    uint32_t f[W];
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+      M[k] = ~M[k] & vx & (vy >> k);  // E[k]
+      f[k] = k == up ? 1u : 0u;
+    }
+#pragma unroll
+    for (int e = 0; e <= T; ++e) {
+      uint32_t at = 0;
+#pragma unroll
+      for (int k = 0; k < W; ++k) {
+        f[k] = (f[k] + M[k]) & ~M[k];
+        if (k == kres) at = f[k];
+      }
+      cells += W;
+      if (at >= goal) {
+        res = e;
+        break;
+      }
+      uint32_t below = 0;
+#pragma unroll
+      for (int k = 0; k < W; ++k) {
+        const uint32_t here = f[k];
+        const uint32_t above = k + 1 < W ? f[k + 1] : 0u;
+        f[k] = max(max(here, above) << 1, below);
+        below = here;
+      }
+    }
+  }
+  return res;
+}
+
+// One side of a match in bit planes: the strings and where the match lies.
+struct PlaneMatch {
+  uint32_t X[8], Y[8];  // probe, indexed string
+  int ls, lr;           // their lengths
+  int p, P, li;         // substring and segment starts, their length
+  int tau, i;
+  bool wide;            // planes 6 and 7 in use
+};
+
+// The side's distance if it is at most its threshold (i - 1 on the left, tau
+// + 1 - i on the right), else a larger value; MAXT: the largest threshold.
+template <int MAXT>
+__host__ __device__ __forceinline__ int plane_side(const PlaneMatch& m, bool right, unsigned& cells) {
+  const int t = right ? m.tau + 1 - m.i : m.i - 1;
+  const int sx = right ? m.p + m.li : 0, nx = right ? m.ls - sx : m.p;
+  const int sy = right ? m.P + m.li : 0, ny = right ? m.lr - sy : m.P;
+  int d = PLANE_LEN;
+  if (t == 0) d = plane_distance<0>(m.X, sx, nx, m.Y, sy, ny, m.wide, cells);
+  else if (t == 1 && MAXT >= 1) d = plane_distance<(MAXT >= 1 ? 1 : 0)>(m.X, sx, nx, m.Y, sy, ny, m.wide, cells);
+  else if (t == 2 && MAXT >= 2) d = plane_distance<(MAXT >= 2 ? 2 : 0)>(m.X, sx, nx, m.Y, sy, ny, m.wide, cells);
+  else if (t == 3 && MAXT >= 3) d = plane_distance<(MAXT >= 3 ? 3 : 0)>(m.X, sx, nx, m.Y, sy, ny, m.wide, cells);
+  else if (t == 4 && MAXT >= 4) d = plane_distance<(MAXT >= 4 ? 4 : 0)>(m.X, sx, nx, m.Y, sy, ny, m.wide, cells);
+  return d;
+}
+
+// Whether substring and segment are equal (a hash collision otherwise).
+__host__ __device__ __forceinline__ bool plane_segment(const PlaneMatch& m) {
+  uint32_t diff = 0;
+#pragma unroll
+  for (int b = 0; b < 8; ++b) diff |= (m.X[b] >> m.p) ^ (m.Y[b] >> m.P);
+  return (diff & ((1u << m.li) - 1u)) == 0;
+}
 
 // Extension-based verification of one match (Sec. 5.2, Alg. 3).  s has the
 // selected substring at p; r is the indexed string whose segment i (start P,

@@ -212,3 +212,17 @@ def test_fused_work_items_cover_every_probe_once(tmp_path):
     out = subprocess.run([str(exe)], capture_output=True, text=True).stdout.strip()
     assert out == f"ok {4 * 300 * 40}", out
 
+
+
+def test_plane_verification_matches_dp(tmp_path):
+    """Bit-plane sides (distance, segment, screen limits) against the plain DP."""
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    exe = str(tmp_path / "plane_check")
+    subprocess.run([nvcc, "-std=c++17", "-O2", "-I", CSRC, "-I", os.path.join(ROOT, "include"), "-o", exe,
+                    os.path.join(ROOT, "tests", "host_logic", "plane_check.cu")], check=True)
+    out = subprocess.run([exe], capture_output=True, text=True, check=True).stdout
+    vals = dict(t.split("=") for t in out.split("\n")[-2].split())
+    assert int(vals["bad"]) == 0, out
+    assert int(vals["within"]) > 10000 and int(vals["sides"]) > 100000
