@@ -104,7 +104,8 @@ typedef struct {
   uint64_t dp_cells;    /* DP cells evaluated by the verification kernels */
   uint64_t fallback_pairs; /* pairs verified directly because a string has length <= tau */
   uint64_t hits;        /* lookups whose posting run was non-empty */
-  float probe_ms;       /* device time of selection + lookup (CUDA events on the call's stream) */
+  float probe_ms;       /* device time of selection + lookup (CUDA events on the call's stream); 0 for a
+                           query batch, whose one kernel does both */
   float verify_ms;      /* device time of extension verification */
   float fallback_ms;    /* device time of the short-string verification */
   float dedupe_ms;      /* device time of sort, min-reduce and compaction */

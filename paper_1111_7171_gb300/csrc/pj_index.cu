@@ -764,6 +764,12 @@ Partition& ensure_partition(pj_index& idx, int tau, float* ms) {
   return part;
 }
 
+void query_planes(const Ctx& c, const pj_index& idx, const ProbeSet& R, Planes* out) {
+  k_planes<<<std::min<unsigned>(ceil_div(R.n, 128), sm_grid_cap(16)), 128, 0, c.stream>>>(R.bytes, R.off, R.n, nullptr,
+                                                                                         idx.byte_bits, out);
+  PJ_LAUNCHED("k_planes");
+}
+
 void upload_probe_set(const Ctx& c, const pj_index& idx, const pj_strings& R, ProbeSet& out, bool planes) {
   const uint8_t* dbytes = nullptr;
   const uint64_t* doff = nullptr;
@@ -794,15 +800,13 @@ void upload_probe_set(const Ctx& c, const pj_index& idx, const pj_strings& R, Pr
   if (R.n) {
     k_signatures<<<std::min<unsigned>(ceil_div(R.n, 256), sm_grid_cap(8)), 256, 0, c.stream>>>(dbytes, doff, R.n, out.bm.p);
     PJ_LAUNCHED("k_signatures");
-    if (planes && idx.splanes.p) {
-      out.planes.reset(c, R.n);
-      k_planes<<<std::min<unsigned>(ceil_div(R.n, 128), sm_grid_cap(16)), 128, 0, c.stream>>>(
-          dbytes, doff, R.n, nullptr, idx.byte_bits, out.planes.p);
-      PJ_LAUNCHED("k_planes");
-    }
   }
   out.bytes = dbytes;
   out.off = doff;
+  if (planes && idx.splanes.p && R.n) {
+    out.planes.reset(c, R.n);
+    query_planes(c, idx, out, out.planes.p);
+  }
   out.own_bytes = std::move(bb);
   out.own_off = std::move(ob);
 }

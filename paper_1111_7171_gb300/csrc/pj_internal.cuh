@@ -406,7 +406,9 @@ __host__ __device__ __forceinline__ int popcount64(unsigned long long x) {
 // about 2 cycles per warp here, against 8.8 for a popcount).
 __host__ __device__ __forceinline__ unsigned byte_distance(uint32_t x, uint32_t y, unsigned acc) {
 #ifdef __CUDA_ARCH__
-  return __vsadu4(x, y) + acc;
+  unsigned r;
+  asm("vabsdiff4.u32.u32.u32.add %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(y), "r"(acc));
+  return r;
 #else
   for (int k = 0; k < 32; k += 8) {
     const int a = (int)(x >> k & 255u), b = (int)(y >> k & 255u);
@@ -595,6 +597,9 @@ struct ProbeSet {
 };
 // planes: with bit planes if idx has them.
 void upload_probe_set(const Ctx& c, const pj_index& idx, const pj_strings& R, ProbeSet& out, bool planes = true);
+
+// Bit planes of R's strings for idx (which has them).
+void query_planes(const Ctx& c, const pj_index& idx, const ProbeSet& R, Planes* out);
 
 // R != S probe of a resident index where probe q has threshold h_tau[q]
 // (host array).  Every threshold present must be built.  Work is ordered on

@@ -39,27 +39,11 @@
 #include "pj_plan.cuh"
 #include "pj_prims.cuh"
 #include "pj_probe.cuh"
+#include "pj_screen.cuh"
 
 namespace pj {
 
 namespace cg = cooperative_groups;
-
-struct Counters {
-  unsigned long long accepted;
-  unsigned long long lookups;
-  unsigned long long candidates;
-  unsigned long long cells;
-  unsigned long long fallback;
-  unsigned long long hits;
-  unsigned long long err;  // bit 0: run or posting outside the index; bit 1: probe limit
-  unsigned long long filtered;  // candidates rejected by the character-count bound
-};
-
-struct AccOut {
-  unsigned long long* key;
-  uint32_t* ed;
-  unsigned long long cap;
-};
 
 constexpr int BLOCK = 256;
 
@@ -68,10 +52,6 @@ constexpr int BLOCK = 256;
 // prefix sums.  (Earlier forms that placed shuffles, ballots or
 // __syncthreads right after the divergent verification loops lost the
 // contributions of lanes still inside those loops.)
-
-__device__ __forceinline__ void add_counter(unsigned long long* c, unsigned long long v) {
-  if (v) atomicAdd(c, v);
-}
 
 // ---------------------------------------------------------------- A4 ------
 
@@ -132,12 +112,6 @@ __device__ __forceinline__ bool group_of(const ProbeView& v, unsigned long long 
     vt = v;
     return local < v.pcount;
   }
-}
-
-// Sizes that a kernel reads from device memory when it starts: the launch
-// covers a capacity `cap`, n_dev (if not NULL) holds the actual count.
-__device__ __forceinline__ unsigned long long dev_count(unsigned long long cap, const unsigned long long* n_dev) {
-  return n_dev ? min(cap, *n_dev) : cap;
 }
 
 // The hit of candidate c: the last hit whose first candidate is <= c
@@ -395,14 +369,6 @@ __global__ void __launch_bounds__(512) k_verify_hits(const ProbeView v, const Hi
 // warps' DP lanes stay full.  The ballots and the queue loop run the same
 // number of times in all 32 lanes, and queue entries are read before the
 // next writes only after a __syncwarp.
-constexpr int Q_BLOCK = 256;
-constexpr int Q_WARPS = Q_BLOCK / 32;
-constexpr int S_RUN = 8;                 // candidates one lane screens per step
-constexpr int Q_CAP = 32 * S_RUN + 32;   // < 32 left + up to 32 * S_RUN new
-constexpr int Q_SECOND = 64;             // < 32 left + up to 32 new
-constexpr unsigned long long Q_CHUNK = 8ull * 32 * S_RUN;  // candidates a warp takes at a time
-constexpr unsigned long long Q_CHUNK_MIN = 128;            // ... in launches too small to fill the warps
-
 // Chunk of a queued verification launch over n candidates by n_warps warps:
 // Q_CHUNK, times up to 4 when every warp gets at least 512 chunks of that
 // size (measured on 2.2e10 candidates: 3% less time with 4; on 3e8, where a
@@ -434,119 +400,6 @@ __device__ __forceinline__ void lane_hit_set(const Hit* __restrict__ hits, uint3
   lh.pi = hit.pi;
   lh.lim = hit.lim;
   lh.sides = hit.sides;
-}
-
-// Extension verification of one queue entry: probe q, indexed sid r, and
-// the match's position, segment and threshold packed in pi.
-template <int MAXW, bool SELF, bool MULTI>
-__device__ __forceinline__ void verify_queued_entry(const ProbeView& v, uint32_t q, uint32_t r, uint32_t pi,
-                                                    AccOut out, Counters* ctr, unsigned long long& cells) {
-  const ProbeView vt = MULTI ? view_for_tau(v, (int)(pi >> 24)) : v;
-  HitCtx hc;
-  hc.q = q;
-  hc.begin = 0;
-  hc.p = (int)(pi & 0xFFFFu);
-  hc.i = (int)((pi >> 16) & 0xFFu);
-  if (vt.pref) {
-    const unsigned long long ref = vt.pref[q];
-    hc.ls = (int)(ref & 0xFFFFu);
-    hc.s = vt.pbytes + (ref >> 16);
-  } else {
-    hc.ls = (int)vt.plen[q];
-    hc.s = vt.pbytes + vt.poff[q];
-  }
-  unsigned long long key = 0;
-  int ed = 0;
-  if (verify_screened<MAXW>(vt, SELF, hc, r, key, ed, cells)) {
-    const unsigned long long pos = atomicAdd(&ctr->accepted, 1ull);
-    if (pos < out.cap) {
-      out.key[pos] = key;
-      out.ed[pos] = (uint32_t)ed;
-    }
-  }
-}
-
-// A warp's queues in shared memory.  A screened match waits in the first
-// until 32 of them are verified together; with bit planes (short strings, tau
-// <= 4) that is only the side with the smaller threshold, and the matches
-// whose first side passed (its distance in place of the left limit) wait in
-// the second until 32 of them can have the other side verified: most matches
-// fail on the first side, and lanes with nothing left to do would idle through
-// the second side's wider band.
-struct SecondQueue {
-  uint32_t q[Q_SECOND], sid[Q_SECOND], pi[Q_SECOND], lim[Q_SECOND];
-};
-struct QueueWarp {
-  uint32_t q[Q_CAP], sid[Q_CAP], pi[Q_CAP], lim[Q_CAP];
-  SecondQueue second;
-};
-
-// First side of one match per lane (`in` lanes have one).  Matches without
-// planes (lengths 0 in lim) are verified as a whole.  n2: the second queue's
-// size, the same in every lane.
-template <int MAXW, bool SELF, bool MULTI>
-__device__ __forceinline__ void verify_first(const ProbeView& v, SecondQueue& w, bool in, uint32_t q, uint32_t r,
-                                             uint32_t pi, uint32_t lim, int& n2, AccOut out, Counters* ctr,
-                                             unsigned long long& cells) {
-  bool pass = false;
-  uint32_t d1 = 0;
-  if (in) {
-    if (MAXW <= 5 && v.pplanes && lim >> 16) {
-      const ProbeView vt = MULTI ? view_for_tau(v, (int)(pi >> 24)) : v;
-      const PlaneMatch m = plane_match(vt, q, r, pi, lim);
-      const int tl = m.i - 1, tr = m.tau + 1 - m.i;
-      unsigned c = 0;
-      if (m.li <= SEG_EXACT_MAX || plane_segment(m)) {
-        const bool right = tr < tl;
-        d1 = (uint32_t)plane_side<(MAXW - 1) / 2>(m, right, c);
-        pass = (int)d1 <= (right ? tr : tl);
-      }
-      cells += c;
-    } else {
-      verify_queued_entry<MAXW, SELF, MULTI>(v, q, r, pi, out, ctr, cells);
-    }
-  }
-  if (MAXW <= 5) {
-    __syncwarp();
-    const unsigned b = __ballot_sync(FULL, pass);
-    if (pass) {
-      const int slot = n2 + __popc(b & lanemask_lt());
-      w.q[slot] = q;
-      w.sid[slot] = r;
-      w.pi[slot] = pi;
-      w.lim[slot] = (lim & ~0xFFu) | d1;
-    }
-    n2 += __popc(b);
-    __syncwarp();
-  }
-}
-
-// Second side of the second queue's last min(n2, 32) entries.
-template <int MAXW, bool SELF, bool MULTI>
-__device__ __forceinline__ void verify_second(const ProbeView& v, SecondQueue& w, int& n2, AccOut out, Counters* ctr,
-                                              unsigned long long& cells) {
-  const int lane = (int)(threadIdx.x & 31u);
-  const int n = ::min(n2, 32);
-  n2 -= n;
-  const int e = n2 + (lane < n ? lane : 0);
-  const uint32_t q = w.q[e], r = w.sid[e], pi = w.pi[e], lim = w.lim[e];
-  __syncwarp();  // taken before any later write
-  if (lane < n) {
-    const ProbeView vt = MULTI ? view_for_tau(v, (int)(pi >> 24)) : v;
-    const PlaneMatch m = plane_match(vt, q, r, pi, lim);
-    const int tl = m.i - 1, tr = m.tau + 1 - m.i;
-    const bool right = !(tr < tl);
-    unsigned c = 0;
-    const int d2 = plane_side<MAXW - 1>(m, right, c);
-    cells += c;
-    if (d2 <= (right ? tr : tl)) {
-      const unsigned long long pos = atomicAdd(&ctr->accepted, 1ull);
-      if (pos < out.cap) {
-        out.key[pos] = match_key(v, SELF, q, r);
-        out.ed[pos] = (lim & 0xFFu) + (uint32_t)d2;
-      }
-    }
-  }
 }
 
 // chunk: candidates a warp takes at a time (0: from the device's count).
@@ -679,20 +532,16 @@ struct __align__(16) Tile {
 };
 
 // Hits per run (cnt, by the run's first posting), each hit's rank among them,
-// and the longest of their counts; totals[0] the candidates.
+// and the longest of their counts.
 __global__ void __launch_bounds__(BLOCK) k_run_count(const Hit* __restrict__ hits, unsigned long long n,
                                                      uint32_t* __restrict__ cnt, uint32_t* __restrict__ longest,
-                                                     uint32_t* __restrict__ rank, unsigned long long* totals) {
-  unsigned long long cand = 0;
+                                                     uint32_t* __restrict__ rank) {
   for (unsigned long long h = (unsigned long long)blockIdx.x * BLOCK + threadIdx.x; h < n;
        h += (unsigned long long)gridDim.x * BLOCK) {
     const uint4 a = *reinterpret_cast<const uint4*>(hits + h);  // q, begin, count, pi
     rank[h] = atomicAdd(&cnt[a.y], 1u);
     if (longest[a.y] < a.z) atomicMax(&longest[a.y], a.z);
-    cand += a.z;
   }
-  cand = warp_sum(cand);
-  if ((threadIdx.x & 31) == 0) add_counter(totals, cand);
 }
 
 __global__ void __launch_bounds__(BLOCK) k_run_scatter(const Hit* __restrict__ hits, unsigned long long n,
@@ -713,7 +562,7 @@ __device__ __forceinline__ unsigned long long run_tiles(uint32_t hits, uint32_t 
          ((posts + (unsigned long long)TILE_POSTS - 1) / TILE_POSTS);
 }
 
-// totals[1]: the tiles of all runs.
+// totals[0]: the tiles of all runs.
 __global__ void __launch_bounds__(BLOCK) k_tile_count(const uint32_t* __restrict__ cnt,
                                                       const uint32_t* __restrict__ longest, unsigned long long n,
                                                       unsigned long long* totals) {
@@ -722,10 +571,10 @@ __global__ void __launch_bounds__(BLOCK) k_tile_count(const uint32_t* __restrict
        b += (unsigned long long)gridDim.x * BLOCK)
     if (cnt[b]) t += run_tiles(cnt[b], longest[b]);
   t = warp_sum(t);
-  if ((threadIdx.x & 31) == 0) add_counter(totals + 1, t);
+  if ((threadIdx.x & 31) == 0) add_counter(totals, t);
 }
 
-// The tiles, in no particular order (totals[2] counts them).
+// The tiles, in no particular order (totals[1] counts them).
 __global__ void __launch_bounds__(BLOCK) k_tile_emit(const uint32_t* __restrict__ cnt,
                                                      const uint32_t* __restrict__ longest,
                                                      const uint32_t* __restrict__ off, unsigned long long n,
@@ -740,7 +589,7 @@ __global__ void __launch_bounds__(BLOCK) k_tile_emit(const uint32_t* __restrict_
     const unsigned long long t = c ? run_tiles(c, m) : 0ull;
     const unsigned long long incl = warp_incl_scan(t);
     unsigned long long at = 0;
-    if (lane == 31 && incl) at = atomicAdd(totals + 2, incl);
+    if (lane == 31 && incl) at = atomicAdd(totals + 1, incl);
     at = __shfl_sync(FULL, at, 31) + incl - t;
     if (t) {
       const uint32_t h0 = off[b];
@@ -811,8 +660,9 @@ __global__ void __launch_bounds__(T_BLOCK) k_screen_tiles(const ProbeView v, con
         const uint4 rec = *reinterpret_cast<const uint4*>(v.precs + tile.x + min(k, posts - 1));
         const bool valid = rec.x < v.n_index;
         if (!valid) err |= 1;
-        sid[j] = k < posts && valid ? rec.x : NO_HIT;
-        L[j][0] = rec.y & SIDE_MASK;
+        sid[j] = rec.x;
+        // a place without a posting: counts that pass no limit (at most 64)
+        L[j][0] = k < posts && valid ? rec.y & SIDE_MASK : 0xFFFFFFFFu;
         L[j][1] = rec.z & SIDE_MASK;
         L[j][2] = rec.w & SIDE_MASK;
         R[j][0] = rec.y >> 4 & SIDE_MASK;
@@ -834,7 +684,7 @@ __global__ void __launch_bounds__(T_BLOCK) k_screen_tiles(const ProbeView v, con
           if (j < nj) {
             const unsigned dl = byte_distance(L[j][2], l2, byte_distance(L[j][1], l1, byte_distance(L[j][0], l0, 0)));
             const unsigned dr = byte_distance(R[j][2], r2, byte_distance(R[j][1], r1, byte_distance(R[j][0], r0, 0)));
-            const bool pass = dl <= bl && dr <= br && lane + 32u * j < mine && sid[j] != NO_HIT;
+            const bool pass = dl <= bl && dr <= br && lane + 32u * j < mine;
             const unsigned m = __ballot_sync(FULL, pass);
             if (pass) w[qn + __popc(m & lanemask_lt())] = make_uint2(h, sid[j]);
             qn += __popc(m);
@@ -1765,15 +1615,20 @@ static void launch_verify(const Ctx& c, const ProbeView& v, const Hit* hits, con
   PJ_LAUNCHED("k_verify_hits");
 }
 
-// Hits from which a chunk is grouped by run and verified tile by tile
-// (PJ_TILES_MIN_HITS overrides).
-constexpr unsigned long long TILES_MIN_HITS = 1ull << 16;
+// Hits, and candidates per hit, from which a chunk is grouped by run and
+// verified tile by tile (PJ_TILES_MIN_HITS overrides the first and drops the
+// second).  Probe + verification, tiles / queued, by candidates per hit: 27
+// (417k short strings, tau 2) 1.39 / 1.25 ms, 50 (200k, tau 3) 1.82 / 1.95, 54
+// (1M, tau 2) 3.22 / 2.93, 64 (100k, tau 4) 1.93 / 2.30, 92 (417k, tau 3) 4.3 /
+// 5.4, 521 (1M, tau 4) 95 / 138 ms.
+constexpr unsigned long long TILES_MIN_HITS = 1ull << 20;
+constexpr unsigned long long TILES_MIN_RUN = 60;
 
 // The hits of a chunk grouped by posting run, and the tiles over them.
 struct HitTiles {
   DBuf<Hit> hits;
   DBuf<Tile> tiles;
-  DBuf<unsigned long long> totals;  // candidates, tiles, tiles written
+  DBuf<unsigned long long> totals;  // tiles, tiles written
   unsigned long long n_tiles = 0;   // 0: not grouped
   // one tile range's survivors
   DBuf<uint2> list;
@@ -1956,6 +1811,7 @@ struct AcceptBuf {
   DBuf<uint32_t> ed;
   unsigned long long cap = 0;
   unsigned long long last = 0;  // accepted count after the last run()
+  bool fresh = false;  // the counters are still zero: the next run() need not read them
   AcceptBuf(const Ctx& ctx, Counters* counters, unsigned long long initial) : c(ctx), ctr(counters) {
     key.reset(c, initial);
     ed.reset(c, initial);
@@ -1973,8 +1829,11 @@ struct AcceptBuf {
   template <class Launch, class Want>
   void run(Launch launch, Want want) {
     Counters saved{};  // all counters, so that a re-run launch is counted once
-    PJ_CUDA(cudaMemcpyAsync(&saved, ctr, sizeof(saved), cudaMemcpyDeviceToHost, c.stream));
-    c.sync();
+    if (!fresh) {
+      PJ_CUDA(cudaMemcpyAsync(&saved, ctr, sizeof(saved), cudaMemcpyDeviceToHost, c.stream));
+      c.sync();
+    }
+    fresh = false;
     const unsigned long long before = saved.accepted;
     launch(out());
     const unsigned long long after = read_count();
@@ -2005,19 +1864,18 @@ struct AcceptBuf {
   }
 };
 
-// Groups n hits over the postings [0, n_postings) of v's index; returns the
-// number of candidates.
-static unsigned long long group_hits(const Ctx& c, const ProbeView& v, DBuf<Hit>& hits, unsigned long long n,
+// Groups n hits over the postings [0, n_postings) of v's index.
+static void group_hits(const Ctx& c, const ProbeView& v, DBuf<Hit>& hits, unsigned long long n,
                                      HitTiles& t) {
   const unsigned long long np = v.n_postings;
   DBuf<uint32_t> cnt(c, 2 * np), off(c, np), rank(c, n);
   uint32_t* longest = cnt.p + np;
-  t.totals.reset(c, 3);
+  t.totals.reset(c, 2);
   PJ_CUDA(cudaMemsetAsync(cnt.p, 0, cnt.bytes(), c.stream));
   PJ_CUDA(cudaMemsetAsync(t.totals.p, 0, t.totals.bytes(), c.stream));
   const unsigned gh = (unsigned)std::min<unsigned long long>((n + BLOCK - 1) / BLOCK, sm_grid_cap(8));
   const unsigned gp = (unsigned)std::min<unsigned long long>((np + BLOCK - 1) / BLOCK, sm_grid_cap(8));
-  k_run_count<<<gh, BLOCK, 0, c.stream>>>(hits.p, n, cnt.p, longest, rank.p, t.totals.p);
+  k_run_count<<<gh, BLOCK, 0, c.stream>>>(hits.p, n, cnt.p, longest, rank.p);
   PJ_LAUNCHED("k_run_count");
   k_tile_count<<<gp, BLOCK, 0, c.stream>>>(cnt.p, longest, np, t.totals.p);
   PJ_LAUNCHED("k_tile_count");
@@ -2025,15 +1883,12 @@ static unsigned long long group_hits(const Ctx& c, const ProbeView& v, DBuf<Hit>
   t.hits.reset(c, n);
   k_run_scatter<<<gh, BLOCK, 0, c.stream>>>(hits.p, n, off.p, rank.p, t.hits.p);
   PJ_LAUNCHED("k_run_scatter");
-  unsigned long long h[2] = {0, 0};
-  PJ_CUDA(cudaMemcpyAsync(h, t.totals.p, sizeof(h), cudaMemcpyDeviceToHost, c.stream));
+  PJ_CUDA(cudaMemcpyAsync(&t.n_tiles, t.totals.p, sizeof(t.n_tiles), cudaMemcpyDeviceToHost, c.stream));
   c.sync();
-  t.n_tiles = h[1];
   t.tiles.reset(c, t.n_tiles);
   k_tile_emit<<<gp, BLOCK, 0, c.stream>>>(cnt.p, longest, off.p, np, t.tiles.p, t.n_tiles, t.totals.p);
   PJ_LAUNCHED("k_tile_emit");
   hits.release();
-  return h[0];
 }
 
 // Probe + verify for all probing strings, in chunks of probing strings whose
@@ -2067,11 +1922,6 @@ static void probe_chunk(const Ctx& c, const ProbeView& v, unsigned long long n_g
                                                         n_hits);
   PJ_LAUNCHED("k_group_hits");
   trace_mark(c, "join: probe (hits)");
-  if (tiles && n_hits >= env_knob("PJ_TILES_MIN_HITS", TILES_MIN_HITS)) {
-    n_cand = group_hits(c, v, hits, n_hits, *tiles);
-    trace_mark(c, "join: group hits by run");
-    return;
-  }
   cnt.reset(c, n_hits + 1);
   off.reset(c, n_hits + 1);
   PJ_CUDA(cudaMemsetAsync(cnt.p + n_hits, 0, sizeof(unsigned long long), c.stream));
@@ -2080,6 +1930,13 @@ static void probe_chunk(const Ctx& c, const ProbeView& v, unsigned long long n_g
   exclusive_scan<unsigned long long>(c, cnt.p, off.p, n_hits + 1);
   PJ_CUDA(cudaMemcpyAsync(&n_cand, off.p + n_hits, sizeof(n_cand), cudaMemcpyDeviceToHost, c.stream));
   c.sync();
+  const unsigned long long knob = env_knob("PJ_TILES_MIN_HITS", 0);
+  if (tiles && (knob ? n_hits >= knob : n_hits >= TILES_MIN_HITS && n_cand >= TILES_MIN_RUN * n_hits)) {
+    cnt.release();
+    off.release();
+    group_hits(c, v, hits, n_hits, *tiles);
+    trace_mark(c, "join: group hits by run");
+  }
 }
 
 // The warp cut-over probe rounded up to the chunk's next probe-block boundary
@@ -2335,6 +2192,25 @@ static bool fused_self_join(const Ctx& c, const ProbeView& v, AcceptBuf& acc, Co
   return true;
 }
 
+// Groups up to which a query batch runs in one launch (k_query_fused); a larger
+// R != S join takes the probe passes, whose lanes roll a window's keys.
+constexpr unsigned long long QUERY_FUSED_MAX_GROUPS = 1ull << 18;
+
+// Room for the parts of a batch's long runs: 8 MiB.
+constexpr unsigned long long QUERY_TASKS = 1ull << 18;
+
+template <int MAXW, bool MULTI>
+static void launch_query(const Ctx& c, const ProbeView& v, unsigned long long n_groups,
+                         const unsigned long long* n_dev, Hit* tasks, unsigned long long task_cap, AccOut out,
+                         Counters* ctr) {
+  const unsigned grid = persistent_grid(k_query_fused<MAXW, MULTI>, (n_groups + Q_WARPS - 1) / Q_WARPS, Q_BLOCK);
+  k_query_fused<MAXW, MULTI><<<grid, Q_BLOCK, 0, c.stream>>>(v, n_groups, n_dev, tasks, task_cap, out, ctr);
+  PJ_LAUNCHED("k_query_fused");
+  const unsigned gt = persistent_grid(k_query_tasks<MAXW, MULTI>, (task_cap + Q_WARPS - 1) / Q_WARPS, Q_BLOCK);
+  k_query_tasks<MAXW, MULTI><<<gt, Q_BLOCK, 0, c.stream>>>(v, tasks, task_cap, out, ctr);
+  PJ_LAUNCHED("k_query_tasks");
+}
+
 template <bool SELF, bool MULTI>
 static void probe_and_verify(const Ctx& c, const ProbeView& v0, uint32_t fb_count, AcceptBuf& acc, Counters* ctr,
                              Counters& h, Timings& tm, const unsigned long long* h_qgoff) {
@@ -2356,7 +2232,7 @@ static void probe_and_verify(const Ctx& c, const ProbeView& v0, uint32_t fb_coun
   const bool use_tiles = !MULTI && !v0.pair_mode && v0.queued && v0.hit_sides && !c.budget &&
                          (uint64_t)v0.warp_q_cut >= (uint64_t)v0.pbegin + v0.pcount;
   unsigned long long total_cand = 0, verified = 0, tile_cand = 0;
-  bool fused_done = false;
+  bool fused_done = false, query_done = false;
   ProbeView vc = v0;  // the probes of the chunked pipeline
   if (SELF && !MULTI && v0.fused && v0.pcount) {  // the fused persistent kernel over the probes from fused_q_cut
     const uint32_t end = v0.pbegin + v0.pcount;
@@ -2366,6 +2242,25 @@ static void probe_and_verify(const Ctx& c, const ProbeView& v0, uint32_t fb_coun
     vf.pcount = end - qf;
     fused_done = vf.pcount > 0 && fused_self_join(c, vf, acc, ctr, tm);
     if (fused_done) vc.pcount = qf - v0.pbegin;
+  }
+  if constexpr (!SELF) {  // a query batch: everything up to the accepted matches in one launch
+    const unsigned long long groups = MULTI ? h_qgoff[v0.pbegin + v0.pcount] : (unsigned long long)v0.pcount * G;
+    if (v0.queued && !v0.pair_mode && groups && groups <= std::min(QUERY_FUSED_MAX_GROUPS, group_budget)) {
+      DBuf<Hit> tasks(c, c.budget ? 1 : QUERY_TASKS);
+      tv.start();
+      acc.fresh = true;  // nothing has run before it
+      acc.run(
+          [&](AccOut o) {
+#define PJ_CALL(W) launch_query<W, MULTI>(c, v0, groups, nullptr, tasks.p, c.budget ? 0 : QUERY_TASKS, o, ctr)
+            PJ_BY_TAU(v0.tau, PJ_CALL);
+#undef PJ_CALL
+          },
+          [&](unsigned long long after) { return 2 * after; });
+      tv.stop();
+      tm.verify += tv.ms();
+      query_done = true;
+      vc.pcount = 0;
+    }
   }
   for (uint32_t done = 0; done < vc.pcount;) {
     ProbeView v = vc;
@@ -2539,10 +2434,10 @@ static void probe_and_verify(const Ctx& c, const ProbeView& v0, uint32_t fb_coun
   PJ_CUDA(cudaMemcpyAsync(&h, ctr, sizeof(Counters), cudaMemcpyDeviceToHost, c.stream));
   c.sync();
   // the chunked pipeline counts candidates and hits on the host, the fused
-  // kernel its candidates on the device
+  // self join its candidates and the query kernel both on the device
   h.filtered += tile_cand;  // the tiles took their survivors off
-  h.candidates = cand + (fused_done ? h.candidates : 0ull);
-  h.hits = nh;
+  h.candidates = cand + (fused_done || query_done ? h.candidates : 0ull);
+  if (!query_done) h.hits = nh;
   if (h.err)
     fail(PJ_ECUDA, std::string("segment index consistency check failed (") +
                        ((h.err & 1) ? "posting outside the index" : "probe limit reached") + ")");
@@ -3362,7 +3257,7 @@ static std::shared_ptr<SelfPlan> make_self_plan(pj_index& idx, const ProbeView& 
   P->cap_acc = std::min<unsigned long long>(0xFFFFFFFFull, with_slack(st.accepted));
   P->cap_pairs = with_slack(pairs);
   const Ctx& c = P->ctx;
-  P->counters.reset(c, 64);
+  P->counters.reset(c, PLAN_COUNTER_BYTES);
   P->sizes.reset(c, 1);
   P->nuniq.reset(c, 1);
   P->gcounts.reset(c, n_groups);
@@ -3713,7 +3608,7 @@ void query_multi_impl(const Ctx& c, pj_index& idx, const ProbeSet& R, const uint
 // Overflowing a capacity only drops writes; the totals are still counted and
 // the host reruns with larger buffers.
 
-static_assert(sizeof(Counters) == 64, "plan counters are 64 bytes");
+static_assert(sizeof(Counters) <= PLAN_COUNTER_BYTES, "plan counters");
 
 // Lengths and group counts of the batch; queries past n get 0 groups, so the
 // group offsets of every q >= n equal the total (group_of searches all cap_q).
@@ -3738,8 +3633,8 @@ __global__ void k_plan_finish(const Counters* __restrict__ ctr, const PlanSizes*
                               PlanHeader* header) {
   PlanHeader h;
   h.groups = sizes->groups;
-  h.hits = sizes->hits;
-  h.cands = sizes->cands;
+  h.hits = ctr->hits;
+  h.cands = ctr->candidates;
   h.accepted = ctr->accepted;
   h.pairs = sizes->pairs;
   h.lookups = ctr->lookups;
@@ -3773,31 +3668,16 @@ void record_query_plan(const Ctx& c, const pj_index& idx, const PlanDev& d) {
   PlanSizes* sz = d.sizes;
   PJ_CUDA(cudaMemsetAsync(ctr, 0, sizeof(Counters), c.stream));
 
-  // A4: groups of every query, lookups, hits, candidate offsets
+  // groups of every query
   k_plan_groups<<<stride_grid(d.cap_q), 256, 0, c.stream>>>(d.bytes, d.off, d.tau, d.cap_q, sz, d.len, d.bm, d.planes,
                                                         idx.byte_bits, d.gcnt);
   PJ_LAUNCHED("k_plan_groups");
   exclusive_scan_dn<unsigned long long>(c, d.gcnt, d.qgoff, d.cap_q, nullptr, &sz->groups);
-  const unsigned g1 = persistent_grid(k_group_counts<false, true>, (d.cap_groups + BLOCK - 1) / BLOCK);
-  k_group_counts<false, true><<<g1, BLOCK, 0, c.stream>>>(v, d.cap_groups, d.gcounts, d.gmask, ctr, &sz->groups);
-  PJ_LAUNCHED("k_group_counts");
-  exclusive_scan_dn<uint32_t>(c, d.gcounts, d.goff, d.cap_groups, &sz->groups, &sz->hits);
-  const unsigned g2 = persistent_grid(k_group_hits<false, true>, (d.cap_groups + BLOCK - 1) / BLOCK);
-  k_group_hits<false, true><<<g2, BLOCK, 0, c.stream>>>(v, d.cap_groups, d.gcounts, d.gmask, d.goff, d.hits,
-                                                        &sz->groups, d.cap_hits);
-  PJ_LAUNCHED("k_group_hits");
-  k_hit_counts<<<stride_grid(d.cap_hits), 256, 0, c.stream>>>(d.hits, d.cap_hits, d.hcnt, &sz->hits);
-  PJ_LAUNCHED("k_hit_counts");
-  exclusive_scan_dn<unsigned long long>(c, d.hcnt, d.hoff, d.cap_hits, &sz->hits, &sz->cands);
-
-  // A6 + A8: verification of every candidate, then the short indexed strings
+  // A4 + A6 in one launch, then A8: the short indexed strings
   const AccOut acc{d.acc_key[0], d.acc_ed[0], d.cap_acc};
 #define PJ_CALL(W)                                                                                              \
   do {                                                                                                         \
-    const unsigned gv = persistent_grid(k_verify_queued<W, false, true>, ~0ull >> 8, Q_BLOCK);                  \
-    k_verify_queued<W, false, true><<<gv, Q_BLOCK, 0, c.stream>>>(v, d.hits, d.hoff, d.cap_hits, 0, 0, acc, ctr, \
-                                                                  &sz->hits, 0);                         \
-    PJ_LAUNCHED("k_verify_queued");                                                                            \
+    launch_query<W, true>(c, v, d.cap_groups, &sz->groups, d.tasks, d.task_cap, acc, ctr);                      \
     if (has_short) {                                                                                           \
       const unsigned gf = persistent_grid(k_fallback<W, false, true>, (d.cap_q + BLOCK - 1) / BLOCK);           \
       k_fallback<W, false, true><<<gf, BLOCK, 0, c.stream>>>(v, d.cap_q, acc, ctr, &sz->n);                     \

@@ -18,8 +18,10 @@
 #include <mutex>
 
 #include "pj_internal.cuh"
+#include "pj_plan.cuh"
 #include "pj_prims.cuh"
 #include "pj_probe.cuh"
+#include "pj_screen.cuh"
 
 namespace pj {
 namespace {
@@ -65,11 +67,7 @@ void* bump_alloc(void* ctx, size_t bytes, void*) {
 
 void bump_free(void*, void*, void*) {}
 
-struct NaCounters {
-  unsigned long long accepted, lookups, candidates, cells, fallback, err;
-};
-
-__device__ __forceinline__ void na_append(NaCounters* ctr, unsigned long long* keys, uint32_t* eds,
+__device__ __forceinline__ void na_append(Counters* ctr, unsigned long long* keys, uint32_t* eds,
                                           unsigned long long cap, unsigned long long key, int ed) {
   const unsigned long long pos = atomicAdd(&ctr->accepted, 1ull);
   if (pos < cap) {
@@ -78,46 +76,11 @@ __device__ __forceinline__ void na_append(NaCounters* ctr, unsigned long long* k
   }
 }
 
-// One thread per (query, indexed length, segment) group: lookups of the
-// multi-match window, then extension verification of every posting of each
-// run, all in the thread (no warp collectives, no barriers).
-template <int MAXW>
-__global__ void __launch_bounds__(NA_BLOCK) k_na_probe_verify(const ProbeView v, unsigned long long n_groups,
-                                                              unsigned long long* keys, uint32_t* eds,
-                                                              unsigned long long cap, NaCounters* ctr) {
-  const int G = groups_per_probe(v.tau, false);
-  unsigned long long lookups = 0, cand = 0, cells = 0;
-  int err = 0;
-  for (unsigned long long t = (unsigned long long)blockIdx.x * NA_BLOCK + threadIdx.x; t < n_groups;
-       t += (unsigned long long)gridDim.x * NA_BLOCK) {
-    const uint32_t q = (uint32_t)(t / G);
-    const int ls = (int)v.plen[q];
-    int l, i, P, li, lo, hi;
-    if (!group_window(v, false, q, ls, (int)(t % G), l, i, P, li, lo, hi)) continue;
-    for (int p = lo; p <= hi; ++p) {
-      ++lookups;
-      uint32_t b;
-      const uint32_t c = lookup(v, false, v.pbytes + v.poff[q], ls, q, l, i, p, li, b, err);
-      const Hit h{q, b, c, (uint32_t)p | ((uint32_t)i << 16)};
-      for (uint32_t k = 0; k < c; ++k) {
-        ++cand;
-        unsigned long long key = 0;
-        int ed = 0;
-        if (verify_candidate<MAXW>(v, false, h, k, key, ed, cells, err)) na_append(ctr, keys, eds, cap, key, ed);
-      }
-    }
-  }
-  if (lookups) atomicAdd(&ctr->lookups, lookups);
-  if (cand) atomicAdd(&ctr->candidates, cand);
-  if (cells) atomicAdd(&ctr->cells, cells);
-  if (err) atomicOr(&ctr->err, (unsigned long long)err);
-}
-
 // Indexed strings of length <= tau have no even partition: every query is
 // verified directly against those within the length filter.
 template <int MAXW>
 __global__ void __launch_bounds__(NA_BLOCK) k_na_fallback(const ProbeView v, unsigned long long* keys, uint32_t* eds,
-                                                          unsigned long long cap, NaCounters* ctr) {
+                                                          unsigned long long cap, Counters* ctr) {
   const int tau = v.tau;
   unsigned long long cells = 0, pairs = 0;
   for (uint32_t x = blockIdx.x * NA_BLOCK + threadIdx.x; x < v.pcount; x += gridDim.x * NA_BLOCK) {
@@ -158,12 +121,17 @@ __global__ void k_na_emit(const unsigned long long* __restrict__ keys, const uin
 
 template <int MAXW>
 void na_launch(const Ctx& c, const ProbeView& v, bool fallback, unsigned long long* keys, uint32_t* eds,
-               unsigned long long cap, NaCounters* ctr) {
+               unsigned long long cap, Hit* tasks, unsigned long long task_cap, Counters* ctr) {
   const unsigned long long n_groups = (unsigned long long)v.pcount * groups_per_probe(v.tau, false);
   if (n_groups) {
-    const unsigned grid = (unsigned)std::min<unsigned long long>((n_groups + NA_BLOCK - 1) / NA_BLOCK, sm_grid_cap(8));
-    k_na_probe_verify<MAXW><<<grid, NA_BLOCK, 0, c.stream>>>(v, n_groups, keys, eds, cap, ctr);
-    PJ_LAUNCHED("k_na_probe_verify");
+    const unsigned grid = (unsigned)std::min<unsigned long long>((n_groups + Q_WARPS - 1) / Q_WARPS, sm_grid_cap(4));
+    const AccOut out{keys, eds, cap};
+    k_query_fused<MAXW, false><<<grid, Q_BLOCK, 0, c.stream>>>(v, n_groups, nullptr, tasks, task_cap, out, ctr);
+    PJ_LAUNCHED("k_query_fused");
+    if (task_cap) {
+      k_query_tasks<MAXW, false><<<sm_grid_cap(4), Q_BLOCK, 0, c.stream>>>(v, tasks, task_cap, out, ctr);
+      PJ_LAUNCHED("k_query_tasks");
+    }
   }
   if (fallback && v.pcount) {
     const unsigned grid = (unsigned)std::min<unsigned>((v.pcount + NA_BLOCK - 1) / NA_BLOCK, sm_grid_cap(8));
@@ -196,8 +164,8 @@ void query_noalloc(pj_index& idx, const pj_strings& batch, int tau, pj_pair* out
 
   ProbeSet R;
   upload_probe_set(c, idx, batch, R, false);  // device input: lengths and signatures only, in the scratch
-  DBuf<NaCounters> ctr(c, 1);
-  PJ_CUDA(cudaMemsetAsync(ctr.p, 0, sizeof(NaCounters), c.stream));
+  DBuf<Counters> ctr(c, 1);
+  PJ_CUDA(cudaMemsetAsync(ctr.p, 0, sizeof(Counters), c.stream));
 
   // Everything left: accepted (key 8 + ed 4), their sort double buffers
   // (12), run flags and positions (8) and the sort histograms.
@@ -207,7 +175,24 @@ void query_noalloc(pj_index& idx, const pj_strings& batch, int tau, pj_pair* out
   DBuf<unsigned long long> keys(c, cap);
   DBuf<uint32_t> eds(c, cap);
 
+  // Bit planes of the queries and room for parts of long runs, when the
+  // scratch has it beside what cap counts on (a match takes at most 36 of its
+  // 40 bytes).
+  DBuf<Planes> planes;
+  DBuf<Hit> tasks;
+  size_t spare = (1u << 20) - (1u << 16) + 4 * cap;
+  if (idx.splanes.p && R.n && align256((size_t)R.n * sizeof(Planes)) <= spare) {
+    planes.reset(c, R.n);
+    query_planes(c, idx, R, planes.p);
+    spare -= align256((size_t)R.n * sizeof(Planes));
+  }
+  if (spare >= (1u << 16)) tasks.reset(c, std::min<size_t>(1u << 16, spare / 2 / sizeof(Hit)));
+
   ProbeView v{};
+  v.pplanes = planes.p;
+  v.iplanes = idx.splanes.p;
+  v.nplanes = planes_used(idx.byte_bits, false);
+  v.hit_sides = part.sides;
   v.ibytes = idx.sbytes.p;
   v.ioff = idx.soff.p;
   v.ilen = idx.slen.p;
@@ -236,7 +221,7 @@ void query_noalloc(pj_index& idx, const pj_strings& batch, int tau, pj_pair* out
   v.pid = nullptr;
   v.key_shift = bits_for(idx.n);
   const bool fallback = part.first > 0;
-#define PJ_NA(W) na_launch<W>(c, v, fallback, keys.p, eds.p, cap, ctr.p)
+#define PJ_NA(W) na_launch<W>(c, v, fallback, keys.p, eds.p, cap, tasks.p, tasks.n, ctr.p)
   if (tau <= 1) PJ_NA(2);
   else if (tau <= 2) PJ_NA(3);
   else if (tau <= 4) PJ_NA(5);
@@ -244,7 +229,7 @@ void query_noalloc(pj_index& idx, const pj_strings& batch, int tau, pj_pair* out
   else if (tau <= 16) PJ_NA(17);
   else PJ_NA(33);
 #undef PJ_NA
-  NaCounters h{};
+  Counters h{};
   PJ_CUDA(cudaMemcpyAsync(&h, ctr.p, sizeof(h), cudaMemcpyDeviceToHost, c.stream));
   c.sync();
   if (h.err) fail(PJ_ECUDA, "pj_query_noalloc: segment index consistency check failed");

@@ -34,13 +34,13 @@ struct pj_plan {
   pj::DBuf<uint8_t> bytes, tau;
   pj::DBuf<uint64_t> off;
   pj::DBuf<pj::PlanSizes> sizes;
-  pj::DBuf<uint32_t> len, gcounts, goff, flags, pos, acc_ed0, acc_ed1;
-  pj::DBuf<unsigned long long> gcnt, qgoff, gmask, hcnt, hoff, acc_key0, acc_key1;
+  pj::DBuf<uint32_t> len, flags, pos, acc_ed0, acc_ed1;
+  pj::DBuf<unsigned long long> gcnt, qgoff, acc_key0, acc_key1;
   pj::DBuf<pj::Sig> bm;
   pj::DBuf<pj::Planes> planes;
   pj::DBuf<pj::PartView> parts;
+  pj::DBuf<pj::Hit> tasks;
   pj::DBuf<unsigned char> counters, arena;
-  pj::DBuf<pj::Hit> hits;
   // pinned host buffers
   pj::HostBuf h_bytes, h_off, h_tau, h_n, h_pairs, h_header;
   cudaGraph_t graph = nullptr;
@@ -49,10 +49,9 @@ struct pj_plan {
   uint64_t runs = 0, captures = 0;
 
   uint64_t device_bytes() const {
-    return bytes.bytes() + tau.bytes() + off.bytes() + sizes.bytes() + len.bytes() + gcounts.bytes() + goff.bytes() +
-           flags.bytes() + pos.bytes() + acc_ed0.bytes() + acc_ed1.bytes() + gcnt.bytes() + qgoff.bytes() +
-           gmask.bytes() + bm.bytes() + planes.bytes() + hcnt.bytes() + hoff.bytes() + acc_key0.bytes() + acc_key1.bytes() + parts.bytes() + counters.bytes() +
-           arena.bytes() + hits.bytes();
+    return bytes.bytes() + tau.bytes() + off.bytes() + sizes.bytes() + len.bytes() + flags.bytes() + pos.bytes() + acc_ed0.bytes() + acc_ed1.bytes() + gcnt.bytes() + qgoff.bytes() +
+           bm.bytes() + planes.bytes() + acc_key0.bytes() + acc_key1.bytes() + parts.bytes() + counters.bytes() +
+           arena.bytes() + tasks.bytes();
   }
   uint64_t host_bytes() const {
     return h_bytes.bytes + h_off.bytes + h_tau.bytes + h_n.bytes + h_pairs.bytes + h_header.bytes;
@@ -70,16 +69,16 @@ struct pj_plan {
     for (auto* b : b8) b->release();
     off.release();
     sizes.release();
-    pj::DBuf<uint32_t>* b32[] = {&len, &gcounts, &goff, &flags, &pos, &acc_ed0, &acc_ed1};
+    pj::DBuf<uint32_t>* b32[] = {&len, &flags, &pos, &acc_ed0, &acc_ed1};
     for (auto* b : b32) b->release();
-    pj::DBuf<unsigned long long>* b64[] = {&gcnt, &qgoff, &gmask, &hcnt, &hoff, &acc_key0, &acc_key1};
+    pj::DBuf<unsigned long long>* b64[] = {&gcnt, &qgoff, &acc_key0, &acc_key1};
     for (auto* b : b64) b->release();
     bm.release();
     planes.release();
     parts.release();
+    tasks.release();
     counters.release();
     arena.release();
-    hits.release();
     if (stream) cudaStreamSynchronize(stream);
     h_bytes.release();
     h_off.release();
@@ -95,16 +94,7 @@ namespace {
 
 constexpr unsigned long long MAX_CAP_ACC = 0xFFFFFFFFull;  // radix sort and u32 positions
 
-// (Re)allocates the capacity-dependent buffers for d's capacities.
-void alloc_hits(pj_plan& P) {
-  P.hits.reset(P.ctx, P.d.cap_hits);
-  P.hcnt.reset(P.ctx, P.d.cap_hits);
-  P.hoff.reset(P.ctx, P.d.cap_hits);
-  P.d.hits = P.hits.p;
-  P.d.hcnt = P.hcnt.p;
-  P.d.hoff = P.hoff.p;
-}
-
+// (Re)allocate the capacity-dependent buffers for d's capacities.
 void alloc_acc(pj_plan& P) {
   P.acc_key0.reset(P.ctx, P.d.cap_acc);
   P.acc_key1.reset(P.ctx, P.d.cap_acc);
@@ -128,8 +118,7 @@ void alloc_pairs(pj_plan& P) {
 // Records the pipeline into a fresh graph and instantiates it.
 void capture(pj_plan& P) {
   P.drop_graph();
-  size_t arena_bytes = scan_temp_bytes(P.d.cap_q) + scan_temp_bytes(P.d.cap_groups) +
-                       scan_temp_bytes(P.d.cap_hits) + scan_temp_bytes(P.d.cap_acc) +
+  size_t arena_bytes = scan_temp_bytes(P.d.cap_q) + scan_temp_bytes(P.d.cap_acc) +
                        sort_temp_bytes(P.d.cap_acc) + (1u << 16);
   for (int attempt = 0;; ++attempt) {
     P.arena.reset(P.ctx, arena_bytes);
@@ -219,6 +208,8 @@ void create(pj_plan& P, pj_index& idx, const pj_plan_options& o) {
   PlanDev& d = P.d;
   d.cap_q = o.max_queries;
   d.cap_groups = cap_groups;
+  // hits take no room since the query kernel keeps none; the capacity only
+  // bounds what a batch may find before the plan is recorded again, as before.
   // defaults: about two hits per group and 128 accepted matches per query
   // (the short-string workload at tau = 4 averages 1.7 and 217 at full
   // self-join scale); capacities grow when a batch needs more
@@ -239,10 +230,10 @@ void create(pj_plan& P, pj_index& idx, const pj_plan_options& o) {
   if (idx.splanes.p) P.planes.reset(P.ctx, d.cap_q);
   P.gcnt.reset(P.ctx, d.cap_q);
   P.qgoff.reset(P.ctx, d.cap_q);
-  P.gcounts.reset(P.ctx, d.cap_groups);
-  P.goff.reset(P.ctx, d.cap_groups);
-  P.gmask.reset(P.ctx, d.cap_groups);
-  P.counters.reset(P.ctx, 64);
+  P.counters.reset(P.ctx, PLAN_COUNTER_BYTES);
+  d.task_cap = std::min<uint64_t>(1u << 18, std::max<uint64_t>(1u << 12, cap_groups));
+  P.tasks.reset(P.ctx, d.task_cap);
+  d.tasks = P.tasks.p;
   d.bytes = P.bytes.p;
   d.off = P.off.p;
   d.tau = P.tau.p;
@@ -252,9 +243,6 @@ void create(pj_plan& P, pj_index& idx, const pj_plan_options& o) {
   d.planes = P.planes.p;
   d.gcnt = P.gcnt.p;
   d.qgoff = P.qgoff.p;
-  d.gcounts = P.gcounts.p;
-  d.goff = P.goff.p;
-  d.gmask = P.gmask.p;
   d.counters = P.counters.p;
   std::vector<PartView> hp((size_t)tau_max + 1);
   for (int t = 0; t <= tau_max; ++t) {
@@ -266,7 +254,6 @@ void create(pj_plan& P, pj_index& idx, const pj_plan_options& o) {
   PJ_CUDA(cudaMemcpyAsync(P.parts.p, hp.data(), hp.size() * sizeof(PartView), cudaMemcpyHostToDevice, P.stream));
   PJ_CUDA(cudaMemsetAsync(P.sizes.p, 0, sizeof(PlanSizes), P.stream));
   d.parts = P.parts.p;
-  alloc_hits(P);
   alloc_acc(P);
   P.h_bytes.reset(o.max_bytes + 16, false);
   P.h_off.reset(((size_t)d.cap_q + 1) * sizeof(uint64_t), false);
@@ -331,7 +318,6 @@ void plan_query(pj_plan& P, const pj_strings& b, const uint8_t* taus, pj_result*
     if (short_of_room && attempt >= 8) fail(PJ_ECUDA, "query plan: capacities still too small after growing");
     if (h.hits > P.d.cap_hits) {
       P.d.cap_hits = grown(P.d.cap_hits, h.hits, P.d.cap_groups * (uint64_t)(tau_max + 1), "hits");
-      alloc_hits(P);
     } else if (h.accepted > P.d.cap_acc) {
       P.d.cap_acc = grown(P.d.cap_acc, h.accepted, MAX_CAP_ACC, "accepted matches");
       alloc_acc(P);

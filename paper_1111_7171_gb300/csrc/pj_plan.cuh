@@ -30,6 +30,8 @@ struct PlanHeader {
   unsigned long long overflow;          // nonzero: a list of the fused self join outgrew its capacity
 };
 
+constexpr size_t PLAN_COUNTER_BYTES = 128;
+
 struct PlanDev {
   uint32_t cap_q;                 // queries per batch
   unsigned long long cap_groups;  // cap_q * groups of the largest threshold
@@ -46,13 +48,9 @@ struct PlanDev {
   unsigned long long* gcnt;       // cap_q groups per query
   unsigned long long* qgoff;      // cap_q group offsets
   const PartView* parts;          // tau_max + 1 thresholds
-  void* counters;                 // 64 bytes, zeroed by the graph
-  uint32_t* gcounts;              // cap_groups
-  uint32_t* goff;                 // cap_groups
-  unsigned long long* gmask;      // cap_groups window-position masks
-  Hit* hits;                      // cap_hits
-  unsigned long long* hcnt;       // cap_hits
-  unsigned long long* hoff;       // cap_hits
+  void* counters;                 // PLAN_COUNTER_BYTES, zeroed by the graph
+  Hit* tasks;                     // task_cap parts of long posting runs
+  unsigned long long task_cap;
   unsigned long long* acc_key[2]; // cap_acc each (sort double buffer)
   uint32_t* acc_ed[2];
   uint32_t* flags;                // cap_acc
