@@ -428,6 +428,73 @@ __global__ void k_table_insert(const unsigned long long* __restrict__ keys, cons
   atomicOr(err, 2);  // table full (cannot happen at load factor <= 1/2)
 }
 
+// The bitmap behind the position masks: (value, segment length) of every
+// distinct key, two bits of one word as in the presence bitmap.
+__global__ void k_value_bits(const unsigned long long* __restrict__ keys, const uint32_t* __restrict__ heads,
+                             uint64_t n_unique, int tau, int scheme, unsigned long long magic, unsigned pb,
+                             unsigned long long mask, uint32_t* __restrict__ bitmap) {
+  const uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (u >= n_unique) return;
+  const unsigned long long key = keys[heads[u]];
+  int P, li;
+  segment_m((int)((key >> 8) & 0xFFFFFFu), tau + 1, magic, scheme, (int)(key & 0xFFu), P, li);
+  if (li <= SEG_EXACT_MAX) return;
+  unsigned long long word;
+  uint32_t bits;
+  presence_of(key_mix(value_key((uint32_t)(key >> 32), li)), mask, pb, word, bits);
+  atomicOr(bitmap + word, bits);
+}
+
+// Position masks of the strings sid first .. n - 1 as probes of the self join:
+// bit p of segment length li says whether some indexed segment of that length
+// has the value of s[p, li) (or a few false ones).  The self join's windows
+// (Sec. 4.2) over the tau + 1 indexed lengths select a position many times --
+// a string of 1,000 at tau 32 has 1,089 windows with about 8,000 positions --
+// but only three segment lengths occur among them, so 3 tests a position
+// stand for all.  One warp per string, a position per lane: the two prefix
+// values are coalesced loads, the bitmap word (16 MB at 100k strings, L2) a
+// scattered one, which bounds the kernel; a ballot makes the mask word.  100k
+// strings of 1,000 at tau 32: 1.09 ms for 2.9e8 tests, and the probe pass that
+// reads the masks 2.35 instead of 5.46 ms (build + join 10.0 -> 8.0 ms).
+__global__ void __launch_bounds__(256) k_position_masks(const uint64_t* __restrict__ soff,
+                                                        const uint32_t* __restrict__ slen,
+                                                        const uint32_t* __restrict__ sph, uint32_t first, uint32_t n,
+                                                        int tau, unsigned pb, unsigned long long mask,
+                                                        const uint32_t* __restrict__ bitmap,
+                                                        uint32_t* __restrict__ pmask) {
+  const unsigned lane = threadIdx.x & 31u;
+  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  for (uint64_t k = first + warp; k < n; k += n_warps) {
+    const int ls = (int)slen[k], base = ls / (tau + 1);
+    const uint32_t* H = sph + soff[k] + k;
+    uint32_t* out = pmask + 3 * mask_word(soff[k], k);
+    uint32_t pw[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) pw[j] = seg_pow(::max(1, base - 1 + j));
+    for (int p0 = 0; p0 < ls; p0 += 32) {
+      const int p = p0 + (int)lane;
+      uint32_t got[3], want[3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const int li = base - 1 + j;
+        got[j] = 0;
+        want[j] = 1;  // no such segment
+        if (li > SEG_EXACT_MAX && p + li <= ls) {
+          unsigned long long word;
+          presence_of(key_mix(value_key(seg_value_from_prefix(H, p, li, pw[j]), li)), mask, pb, word, want[j]);
+          got[j] = bitmap[word];
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const unsigned b = __ballot_sync(FULL, (got[j] & want[j]) == want[j]);
+        if ((int)lane == j) out[3 * (p0 >> 5) + j] = b;
+      }
+    }
+  }
+}
+
 }  // namespace
 
 // Stage a string set on the device (bytes rebased to offset 0).
@@ -584,6 +651,52 @@ constexpr uint64_t SIDES_MAX_AVG_LEN = 256;
 
 void check_partition(const Ctx& c, const Partition& part);
 
+// Positions that the windows of one probe select over all groups of the self
+// join, when nothing clips them.
+static uint64_t window_positions(int tau) {
+  uint64_t sum = 0;
+  for (int D = 0; D <= tau; ++D)
+    for (int a = 0; a <= tau; ++a) {
+      const int b = tau - a;
+      sum += (uint64_t)std::max(0, std::min(a, D + b) + std::min(a, b - D) + 1);
+    }
+  return sum;
+}
+
+// Position masks (k_position_masks) for indexes of long strings, when the
+// windows select a position at least MASKS_MIN_SHARE times for every test that
+// the masks make of it (3 per byte).  Under a device budget, or without
+// memory for them, the join looks every position up.
+constexpr uint64_t MASKS_MIN_SHARE = 2;
+
+static void build_position_masks(const pj_index& idx, Partition& part, const unsigned long long* keys,
+                                 const uint32_t* heads) {
+  const Ctx& c = idx.ctx;
+  if (part.sides || c.budget || !idx.sph.p) return;
+  if (window_positions(part.tau) * idx.n < MASKS_MIN_SHARE * 3 * idx.total_bytes) return;
+  const uint64_t cap = part.table.n;
+  DBuf<uint32_t> bitmap;
+  try {
+    bitmap.reset(c, cap * part.presence_bytes / 4);
+    part.pmask.reset(c, 3 * (mask_word(idx.total_bytes, idx.n) + 1));
+  } catch (const Error& e) {
+    if (e.code != PJ_ENOMEM) throw;
+    bitmap.release();
+    part.pmask.release();
+    return;
+  }
+  PJ_CUDA(cudaMemsetAsync(bitmap.p, 0, bitmap.bytes(), c.stream));
+  k_value_bits<<<ceil_div(part.n_unique, 256), 256, 0, c.stream>>>(keys, heads, part.n_unique, part.tau, part.scheme,
+                                                                   seg_magic(part.tau + 1), part.presence_bytes,
+                                                                   cap - 1, bitmap.p);
+  PJ_LAUNCHED("k_value_bits");
+  const uint32_t np = idx.n - part.first;
+  k_position_masks<<<std::min<unsigned>(ceil_div(np, 8), sm_grid_cap(8)), 256, 0, c.stream>>>(
+      idx.soff.p, idx.slen.p, idx.sph.p, part.first, idx.n, part.tau, part.presence_bytes, cap - 1, bitmap.p,
+      part.pmask.p);
+  PJ_LAUNCHED("k_position_masks");
+}
+
 // Window size of group (length offset, segment i) when nothing clips it
 // (Sec. 4.2): with a = i - 1, b = tau + 1 - i and D = |s| - l the window
 // [max(P - a, P + D - b), min(P + a, P + D + b)] holds
@@ -690,6 +803,7 @@ void build_partition(pj_index& idx, int tau, Partition& part) {
         part.postings.p, keys.p, nrec, part.first, tau, sides.p, part.precs.p);
     PJ_LAUNCHED("k_post_records");
   }
+  build_position_masks(idx, part, keys.p, heads.p);
   trace_mark(c, "partition: table");
   if (getenv("PJ_CHECK_INDEX")) check_partition(c, part);
   if (getenv("PJ_DEBUG_DUMP")) {

@@ -518,6 +518,18 @@ __host__ __device__ __forceinline__ int planes_used(ByteBits bb, bool self) {
   return self || n == 8 ? n : n + 1;
 }
 
+// Position masks: word w (positions 32w .. 32w + 31) of string k, for the
+// segment lengths base - 1, base, base + 1 (base = |s| / (tau + 1)), is
+// pmask[3 * (mask_word(off[k], k) + w)] and the two after it.  A string of n
+// bytes has room for ceil(n / 32) words.
+__host__ __device__ __forceinline__ uint64_t mask_word(uint64_t off, uint64_t k) { return (off >> 5) + k; }
+
+// What the values of all segments of one length, whatever indexed length and
+// segment number they belong to, are known by in the bitmap behind the masks.
+__host__ __device__ __forceinline__ unsigned long long value_key(uint32_t V, int li) {
+  return (unsigned long long)V << 32 | (uint32_t)li;
+}
+
 // One threshold's segment index.
 struct Partition {
   int tau = -1;
@@ -535,6 +547,9 @@ struct Partition {
   // group visiting order for one probe: the (length, segment) groups sorted
   // by window size, widest first; [0] for R != S probes, [1] for the self join
   DBuf<uint16_t> gorder[2];
+  // position masks of the indexed strings as probes of the self join
+  // (k_position_masks; empty: not built)
+  DBuf<uint32_t> pmask;
 };
 
 }  // namespace pj

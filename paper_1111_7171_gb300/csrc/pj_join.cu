@@ -3450,6 +3450,7 @@ static void self_join_impl(pj_index& idx, int tau, pj_result* out, bool on_devic
   v.pplanes = idx.splanes.p;
   v.nplanes = planes_used(idx.byte_bits, true);
   v.phash = idx.sph.p;
+  v.pmask = part.pmask.p;
   v.key_shift = bits_for(idx.n);
   v.gorder = part.gorder[1].p;
   v.warp_q_cut = UINT32_MAX;

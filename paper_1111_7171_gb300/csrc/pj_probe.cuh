@@ -75,6 +75,7 @@ struct ProbeView {
   const uint8_t* table_fp;  // slot fingerprints, then the presence bitmap (NULL: probe the slots directly)
   unsigned table_pb;        // presence bitmap bytes per slot
   const uint32_t* phash;    // probe-side prefix values from poff[q] + q (NULL: computed per window)
+  const uint32_t* pmask;    // probe-side position masks (Partition::pmask; NULL: every position is looked up)
   unsigned long long mask;
   const uint32_t* postings;
   const PostRec* precs;  // postings' records (same order)
@@ -250,9 +251,33 @@ __host__ __device__ __forceinline__ unsigned long long fused_item(unsigned long 
 // instructions, and the batch's extra registers cost occupancy.  Testing the
 // whole window's presence bits first and looking up the passing positions
 // after measured 5% faster on long strings at tau 32 and slower elsewhere.)
+// With position masks the windows of one segment length share a test per
+// position, made once (k_position_masks), instead of one per window.
 template <class F>
 __device__ __forceinline__ void window_lookups(const ProbeView& v, bool self, uint32_t q, int ls, int l, int i, int li,
                                                int lo, int hi, const uint8_t* s, int& err, F f) {
+  if (v.pmask && li > SEG_EXACT_MAX) {  // only the positions whose value some indexed segment of this length has
+    const unsigned k = (unsigned)(li + 1 - (int)(((unsigned long long)(unsigned)ls * v.seg_magic) >> 32));
+    if (k < 3) {
+      const uint32_t* M = v.pmask + 3 * mask_word(v.poff[q], q) + k;
+      const uint32_t* H = v.phash + v.poff[q] + q;
+      uint32_t pw = 0;
+      for (int w = lo >> 5; w <= hi >> 5; ++w) {
+        uint32_t m = M[3 * w];
+        if (w == lo >> 5) m &= ~0u << (lo & 31);
+        if (w == hi >> 5) m &= ~0u >> (31 - (hi & 31));
+        if (m && !pw) pw = seg_pow(li);  // odd, so never 0 once set
+        for (; m; m &= m - 1) {
+          const int p = 32 * w + __ffs((int)m) - 1;
+          uint32_t b;
+          const uint32_t cnt =
+              lookup_key(v, self, q, ls, l, seg_key_of(seg_value_from_prefix(H, p, li, pw), l, i), b, err);
+          if (cnt) f(p, b, cnt);
+        }
+      }
+      return;
+    }
+  }
   const uint32_t pw = seg_pow(li);
   uint32_t V = v.phash && li > SEG_EXACT_MAX ? seg_value_from_prefix(v.phash + v.poff[q] + q, lo, li, pw)
                                              : seg_value(s + lo, li);
