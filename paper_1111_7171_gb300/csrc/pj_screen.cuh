@@ -29,6 +29,13 @@ __device__ __forceinline__ void add_counter(unsigned long long* c, unsigned long
   if (v) atomicAdd(c, v);
 }
 
+// The same by a whole warp, one atomic for its lanes' sum: in a kernel of a few
+// microseconds the counters' atomics on one address are a visible part.
+__device__ __forceinline__ void warp_add_counter(unsigned long long* c, unsigned long long v) {
+  v = warp_sum(v);
+  if ((threadIdx.x & 31u) == 0) add_counter(c, v);
+}
+
 // Sizes that a kernel reads from device memory when it starts: the launch
 // covers a capacity `cap`, n_dev (if not NULL) holds the actual count.
 __device__ __forceinline__ unsigned long long dev_count(unsigned long long cap, const unsigned long long* n_dev) {
@@ -168,6 +175,8 @@ __device__ __forceinline__ void verify_second(const ProbeView& v, SecondQueue& w
 // window.  Bound by the latency of dependent lookups at small batches and by
 // the screen's issue slots at large ones.
 constexpr uint32_t RUN_PART = 256;
+constexpr int STEP_MOST = 512;       // candidates a warp walks itself in one step ...
+constexpr uint32_t RUN_KEEP = 32;    // ... or else only its runs of at most so many
 constexpr int WALK = 4;  // records a lane loads at once
 
 struct WalkWarp {
@@ -286,6 +295,7 @@ __device__ __forceinline__ void walk_runs(const ProbeView& v, WalkWarp& w, WalkS
 // What is left in the queues, and the counters.
 template <int MAXW, bool MULTI>
 __device__ __forceinline__ void walk_end(const ProbeView& v, WalkWarp& w, WalkState& st, AccOut out, Counters* ctr) {
+  __syncwarp();
   if (st.qn) walk_verify<MAXW, MULTI>(v, w, st, st.qn, out, ctr);
   if (MAXW <= 5) {
     while (st.n2) {
@@ -293,8 +303,8 @@ __device__ __forceinline__ void walk_end(const ProbeView& v, WalkWarp& w, WalkSt
       __syncwarp();
     }
   }
-  add_counter(&ctr->cells, st.cells);
-  add_counter(&ctr->filtered, st.filtered);
+  warp_add_counter(&ctr->cells, st.cells);
+  warp_add_counter(&ctr->filtered, st.filtered);
   if (st.err) atomicOr(&ctr->err, (unsigned long long)st.err);
 }
 
@@ -316,7 +326,9 @@ __global__ void __launch_bounds__(Q_BLOCK) k_query_fused(const ProbeView v, unsi
   const unsigned long long n_warps = ((unsigned long long)gridDim.x * Q_BLOCK) >> 5;
   const unsigned W = (unsigned)v.tau + 1;  // the largest window
   const unsigned most = W >= 32 ? 1u : 32u / W;
-  const unsigned per = (unsigned)min((unsigned long long)most, max(1ull, n_groups / n_warps));
+  const unsigned long long rounds = max(1ull, (n_groups + n_warps * most - 1) / (n_warps * most));
+  const unsigned per =  // as many as make the rounds even, rather than a last one for a few warps
+      (unsigned)min((unsigned long long)most, max(1ull, (n_groups + n_warps * rounds - 1) / (n_warps * rounds)));
   unsigned long long lookups = 0, cand = 0, n_hits = 0;
   WalkState st{0ull, 0ull, 0, 0, 0};
   for (unsigned long long t0 = warp * per; t0 < n_groups; t0 += n_warps * per) {
@@ -362,38 +374,55 @@ __global__ void __launch_bounds__(Q_BLOCK) k_query_fused(const ProbeView v, unsi
         }
       }
       __syncwarp();
-      for (unsigned found = __ballot_sync(FULL, mine.count > RUN_PART); found; found &= found - 1) {  // long runs
-        const int src = __ffs((int)found) - 1;
-        Hit hit;
-        hit.q = __shfl_sync(FULL, mine.q, src);
-        hit.begin = __shfl_sync(FULL, mine.begin, src);
-        hit.count = __shfl_sync(FULL, mine.count, src);
-        hit.pi = __shfl_sync(FULL, mine.pi, src);
-        hit.lim = __shfl_sync(FULL, mine.lim, src);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) hit.sides.w[k] = __shfl_sync(FULL, mine.sides.w[k], src);
-        if ((int)lane == src) mine.count = 0;
-        const unsigned long long parts = (hit.count + (unsigned long long)RUN_PART - 1) / RUN_PART;
+      // runs to set aside: the long ones, and in a step of many candidates all
+      // but the shortest, in parts that the whole step reserves at once
+      const int here = warp_sum(mine.count <= RUN_PART ? (int)mine.count : 0);  // the same in every lane
+      const uint32_t cut = task_cap && here > STEP_MOST ? RUN_KEEP : RUN_PART;
+      const bool aside = mine.count > cut;
+      if (__any_sync(FULL, aside)) {
+        const unsigned long long parts = aside ? (mine.count + (unsigned long long)RUN_PART - 1) / RUN_PART : 0ull;
+        const unsigned long long incl = warp_incl_scan(parts);
+        const unsigned long long all = __shfl_sync(FULL, incl, 31);
         unsigned long long at = task_cap;
-        if (lane == 0 && task_cap) at = atomicAdd(&ctr->tasks, parts);
+        if (lane == 0 && task_cap) at = atomicAdd(&ctr->tasks, all);
         at = __shfl_sync(FULL, at, 0);
-        const bool room = at + parts <= task_cap;
-        for (unsigned long long k = lane; k < parts && at + k < task_cap; k += 32) {
-          Hit part = hit;  // empty where not all parts have room
-          part.begin = hit.begin + (uint32_t)k * RUN_PART;
-          part.count = room ? min(RUN_PART, hit.count - (uint32_t)k * RUN_PART) : 0u;
-          tasks[at + k] = part;
+        const bool room = at + all <= task_cap;  // the same in every lane
+        if (parts == 1 && at + incl - 1 < task_cap) {
+          Hit part = mine;
+          if (!room) part.count = 0u;  // empty where not all parts have room
+          tasks[at + incl - 1] = part;
         }
-        __syncwarp();
-        if (!room) walk_run<MAXW, MULTI>(v, w, st, hit, out, ctr);
+        if (parts == 1 && room) mine.count = 0;
+        for (unsigned found = __ballot_sync(FULL, parts > 1); found; found &= found - 1) {  // long runs
+          const int src = __ffs((int)found) - 1;
+          Hit hit;
+          hit.q = __shfl_sync(FULL, mine.q, src);
+          hit.begin = __shfl_sync(FULL, mine.begin, src);
+          hit.count = __shfl_sync(FULL, mine.count, src);
+          hit.pi = __shfl_sync(FULL, mine.pi, src);
+          hit.lim = __shfl_sync(FULL, mine.lim, src);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) hit.sides.w[k] = __shfl_sync(FULL, mine.sides.w[k], src);
+          if ((int)lane == src) mine.count = 0;
+          const unsigned long long np = __shfl_sync(FULL, parts, src);
+          const unsigned long long first = at + __shfl_sync(FULL, incl, src) - np;
+          for (unsigned long long k = lane; k < np && first + k < task_cap; k += 32) {
+            Hit part = hit;
+            part.begin = hit.begin + (uint32_t)k * RUN_PART;
+            part.count = room ? min(RUN_PART, hit.count - (uint32_t)k * RUN_PART) : 0u;
+            tasks[first + k] = part;
+          }
+          __syncwarp();
+          if (!room) walk_run<MAXW, MULTI>(v, w, st, hit, out, ctr);
+        }
       }
       walk_runs<MAXW, MULTI>(v, w, st, mine, out, ctr);
     }
   }
   walk_end<MAXW, MULTI>(v, w, st, out, ctr);
-  add_counter(&ctr->lookups, lookups);
-  add_counter(&ctr->candidates, cand);
-  add_counter(&ctr->hits, n_hits);
+  warp_add_counter(&ctr->lookups, lookups);
+  warp_add_counter(&ctr->candidates, cand);
+  warp_add_counter(&ctr->hits, n_hits);
 }
 
 // The parts that k_query_fused set aside, a warp a part.
