@@ -242,6 +242,16 @@ __global__ void k_signatures(const uint8_t* __restrict__ bytes, const uint64_t* 
     bm[k] = char_signature(bytes + off[k], (int)(off[k + 1] - off[k]));
 }
 
+// The same, a warp each.
+__global__ void k_signatures_warp(const uint8_t* __restrict__ bytes, const uint64_t* __restrict__ off, uint32_t n,
+                                  Sig* __restrict__ bm) {
+  const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  for (uint64_t k = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += n_warps) {
+    const Sig t = warp_signature(bytes + off[k], (int)(off[k + 1] - off[k]));
+    if ((threadIdx.x & 31u) == 0) bm[k] = t;
+  }
+}
+
 // The bits of any and of all of n bytes: orr and ~andd by atomicOr into
 // out[0], out[1] (zero before).
 __global__ void k_byte_bits(const uint8_t* __restrict__ bytes, uint64_t n, uint32_t* __restrict__ out) {
@@ -497,6 +507,26 @@ __global__ void __launch_bounds__(256) k_position_masks(const uint64_t* __restri
 
 }  // namespace
 
+// Character signatures of n strings of `total` bytes.  A thread per string is
+// the cheaper form (its counts need no adding up) while the strings are short
+// and many enough to hide a thread's serial chain; long strings (100k of 1,000
+// bytes: 265 us by threads) and small sets (a batch with queries of 200
+// characters: 14 us) take a warp each.
+constexpr uint64_t SIG_WARP_AVG_LEN = 256;
+constexpr uint32_t SIG_WARP_STRINGS = 1u << 15;
+
+static void launch_signatures(const Ctx& c, const uint8_t* bytes, const uint64_t* off, uint32_t n, uint64_t total,
+                              Sig* bm) {
+  if (n <= SIG_WARP_STRINGS || total > SIG_WARP_AVG_LEN * n) {
+    k_signatures_warp<<<std::min<unsigned>(ceil_div((size_t)n * 32, 256), sm_grid_cap(8)), 256, 0, c.stream>>>(bytes, off,
+                                                                                                              n, bm);
+    PJ_LAUNCHED("k_signatures_warp");
+  } else {
+    k_signatures<<<std::min<unsigned>(ceil_div(n, 256), sm_grid_cap(8)), 256, 0, c.stream>>>(bytes, off, n, bm);
+    PJ_LAUNCHED("k_signatures");
+  }
+}
+
 // Stage a string set on the device (bytes rebased to offset 0).
 static void stage_strings(const Ctx& c, const pj_strings& S, DBuf<uint8_t>& bytes, DBuf<uint64_t>& off,
                           const uint8_t** dbytes, const uint64_t** doff, uint64_t* total) {
@@ -596,9 +626,7 @@ void build_store(pj_index& idx, const pj_strings& S) {
   }
   idx.sbm.reset(c, n ? n : 1);
   if (n) {
-    k_signatures<<<std::min<unsigned>(ceil_div(n, 256), sm_grid_cap(8)), 256, 0, c.stream>>>(idx.sbytes.p, idx.soff.p, n,
-                                                                                    idx.sbm.p);
-    PJ_LAUNCHED("k_signatures");
+    launch_signatures(c, idx.sbytes.p, idx.soff.p, n, total, idx.sbm.p);
   }
   if (total >> 48) fail(PJ_EINVAL, "pj_strings: more than 2^48 bytes");
   idx.sref.reset(c, n ? n : 1);
@@ -912,8 +940,7 @@ void upload_probe_set(const Ctx& c, const pj_index& idx, const pj_strings& R, Pr
   out.lmax = (int)h_lmax;
   out.bm.reset(c, R.n ? R.n : 1);
   if (R.n) {
-    k_signatures<<<std::min<unsigned>(ceil_div(R.n, 256), sm_grid_cap(8)), 256, 0, c.stream>>>(dbytes, doff, R.n, out.bm.p);
-    PJ_LAUNCHED("k_signatures");
+    launch_signatures(c, dbytes, doff, R.n, total, out.bm.p);
   }
   out.bytes = dbytes;
   out.off = doff;

@@ -226,6 +226,38 @@ __host__ __device__ __forceinline__ Sig char_signature(const uint8_t* p, int n) 
   return t;
 }
 
+#ifdef __CUDACC__
+// char_signature by a whole warp (every lane calls it with the same string,
+// and has the result): each lane counts every 32nd character in 4-bit numbers
+// that stop at 4, and the lanes' counts are added, stopping at 4.
+__device__ __forceinline__ Sig warp_signature(const uint8_t* p, int n) {
+  uint32_t c[3] = {0u, 0u, 0u};
+  for (int k = (int)(threadIdx.x & 31u); k < n; k += 32) {
+    const int b = (int)(p[k] % SIG_BUCKETS);
+    const int word = b >> 3, sh = 4 * (b & 7);
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      if (j == word && (c[j] >> sh & 15u) < 4u) c[j] += 1u << sh;
+  }
+  __syncwarp();
+  Sig t = {{0u, 0u, 0u, 0u}};
+  constexpr uint32_t ONES = 0x11111111u;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    uint32_t s = c[j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      s += __shfl_xor_sync(FULL, s, o);  // at most 8 each
+      const uint32_t big = (s >> 2 | s >> 3) & ONES;
+      s = (s & ~(big * 15u)) | big << 2;
+    }
+    t.w[j] = ((s | s >> 1 | s >> 2) & ONES) | ((s >> 1 | s >> 2) & ONES) << 1 | (((s & s >> 1) | s >> 2) & ONES) << 2 |
+             (s >> 2 & ONES) << 3;
+  }
+  return t;
+}
+#endif
+
 __host__ __device__ __forceinline__ int popcount32(uint32_t x) {
 #ifdef __CUDA_ARCH__
   return __popc(x);
@@ -509,6 +541,27 @@ __host__ __device__ __forceinline__ Planes string_planes(const uint8_t* p, int n
   }
   return t;
 }
+
+#ifdef __CUDACC__
+// string_planes by a whole warp: a character per lane, a ballot per plane.
+__device__ __forceinline__ Planes warp_planes(const uint8_t* p, int n, ByteBits bb) {
+  Planes t = {{0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u}};
+  if (n > PLANE_LEN) return t;
+  const uint32_t vary = bb.orr & ~bb.andd & 255u, same = ~vary & 255u;
+  const int lane = (int)(threadIdx.x & 31u);
+  const uint32_t c = lane < n ? p[lane] : 0u;
+  uint32_t v = vary;
+  bool foreign = ((c ^ bb.andd) & same) != 0;
+#pragma unroll
+  for (int b = 0; b < 8; ++b) {
+    const uint32_t low = v & (0u - v);
+    t.w[b] = __ballot_sync(FULL, lane < n && (low ? (c & low) != 0 : foreign));
+    foreign = low ? foreign : false;  // one plane marks it
+    v &= v - 1;
+  }
+  return t;
+}
+#endif
 
 // Planes in use: those of the differing bits and, for probes that are not
 // indexed strings, the marking one.

@@ -3618,15 +3618,21 @@ __global__ void k_plan_groups(const uint8_t* __restrict__ bytes, const uint64_t*
                               uint32_t* __restrict__ len, Sig* __restrict__ bm, Planes* __restrict__ planes,
                               ByteBits bb, unsigned long long* __restrict__ gcnt) {
   const unsigned long long n = sizes->n;
-  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < cap_q; q += gridDim.x * blockDim.x) {
-    if (q < n) {
-      len[q] = (uint32_t)(off[q + 1] - off[q]);
-      bm[q] = char_signature(bytes + off[q], (int)len[q]);
-      if (planes) planes[q] = string_planes(bytes + off[q], (int)len[q], bb);
-      gcnt[q] = (unsigned long long)groups_per_probe((int)tau[q], false);
-    } else {
-      gcnt[q] = 0;
+  const unsigned long long n_warps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
+  for (unsigned long long q = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < cap_q; q += n_warps) {
+    unsigned long long groups = 0;
+    if (q < n) {  // the same in every lane
+      const int l = (int)(off[q + 1] - off[q]);
+      const Sig t = warp_signature(bytes + off[q], l);
+      const Planes pl = planes ? warp_planes(bytes + off[q], l, bb) : Planes{};
+      if ((threadIdx.x & 31u) == 0) {
+        len[q] = (uint32_t)l;
+        bm[q] = t;
+        if (planes) planes[q] = pl;
+      }
+      groups = (unsigned long long)groups_per_probe((int)tau[q], false);
     }
+    if ((threadIdx.x & 31u) == 0) gcnt[q] = groups;
   }
 }
 
@@ -3670,7 +3676,7 @@ void record_query_plan(const Ctx& c, const pj_index& idx, const PlanDev& d) {
   PJ_CUDA(cudaMemsetAsync(ctr, 0, sizeof(Counters), c.stream));
 
   // groups of every query
-  k_plan_groups<<<stride_grid(d.cap_q), 256, 0, c.stream>>>(d.bytes, d.off, d.tau, d.cap_q, sz, d.len, d.bm, d.planes,
+  k_plan_groups<<<stride_grid(32ull * d.cap_q), 256, 0, c.stream>>>(d.bytes, d.off, d.tau, d.cap_q, sz, d.len, d.bm, d.planes,
                                                         idx.byte_bits, d.gcnt);
   PJ_LAUNCHED("k_plan_groups");
   exclusive_scan_dn<unsigned long long>(c, d.gcnt, d.qgoff, d.cap_q, nullptr, &sz->groups);
