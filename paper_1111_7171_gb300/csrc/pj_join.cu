@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(BLOCK) k_group_counts(const ProbeView v, unsig
     counts[t] = nh;
     masks[t] = mask;
   }
-  add_counter(&ctr->lookups, lookups);
+  warp_add_counter(&ctr->lookups, lookups);
   if (err) atomicOr(&ctr->err, (unsigned long long)err);
 }
 
@@ -499,8 +499,8 @@ __global__ void __launch_bounds__(Q_BLOCK) k_verify_queued(const ProbeView v, co
   if (MAXW <= 5) {
     while (n2) verify_second<MAXW, SELF, MULTI>(v, w.second, n2, out, ctr, cells);
   }
-  add_counter(&ctr->cells, cells);
-  add_counter(&ctr->filtered, filtered);
+  warp_add_counter(&ctr->cells, cells);
+  warp_add_counter(&ctr->filtered, filtered);
   if (err) atomicOr(&ctr->err, (unsigned long long)err);
 }
 
@@ -768,7 +768,7 @@ __global__ void __launch_bounds__(T_BLOCK) k_verify_list(const ProbeView v, cons
     verify_second<MAXW, SELF, false>(v, w, n2, out, ctr, cells);
     __syncwarp();
   }
-  add_counter(&ctr->cells, cells);
+  warp_add_counter(&ctr->cells, cells);
 }
 
 // Verification, one thread per entry, of the entries that planes do not
@@ -792,7 +792,7 @@ __global__ void __launch_bounds__(T_BLOCK) k_verify_rest(const ProbeView v, cons
     if (rest && !listed && hits[e.x].lim >> 16) continue;
     verify_queued_entry<MAXW, SELF, false>(v, a.x, e.y, a.w, out, ctr, cells);
   }
-  add_counter(&ctr->cells, cells);
+  warp_add_counter(&ctr->cells, cells);
 }
 
 // One warp per candidate (long strings): the warp walks candidates
@@ -1066,8 +1066,8 @@ __global__ void __launch_bounds__(BLOCK) k_verify_pairs(const ProbeView v, const
       }
     }
   }
-  add_counter(&ctr->cells, cells);
-  add_counter(&ctr->filtered, filtered);
+  warp_add_counter(&ctr->cells, cells);
+  warp_add_counter(&ctr->filtered, filtered);
 }
 
 // Length of the common prefix of a and b (n bytes at most), by the whole
@@ -1451,13 +1451,13 @@ __global__ void __launch_bounds__(FB) k_fused_self(const ProbeView v, int ppi, i
                                 filtered);
     }
   }
-  add_counter(&ctr->lookups, lookups);
-  add_counter(&ctr->candidates, n_cand);
-  add_counter(&ctr->filtered, filtered);
-  add_counter(&work[1], pairs);
+  warp_add_counter(&ctr->lookups, lookups);
+  warp_add_counter(&ctr->candidates, n_cand);
+  warp_add_counter(&ctr->filtered, filtered);
+  warp_add_counter(&work[1], pairs);
   if (err) atomicOr(&ctr->err, (unsigned long long)err);
   // the warp form counts each pair's cells in all 32 lanes: lane 0 reports them
-  add_counter(&ctr->cells, cells + (lane == 0 ? wcells : 0ull));
+  warp_add_counter(&ctr->cells, cells + (lane == 0 ? wcells : 0ull));
 }
 
 // ---------------------------------------------------------------- A8 ------

@@ -29,9 +29,11 @@ __device__ __forceinline__ void add_counter(unsigned long long* c, unsigned long
   if (v) atomicAdd(c, v);
 }
 
-// The same by a whole warp, one atomic for its lanes' sum: in a kernel of a few
-// microseconds the counters' atomics on one address are a visible part.
+// The same by a whole warp, one atomic for its lanes' sum.  An atomic per lane
+// on one address, half a million of them for a full grid with four counters,
+// takes some 100 us: a plan's batch of 64 queries 244 us, 152 us by warps.
 __device__ __forceinline__ void warp_add_counter(unsigned long long* c, unsigned long long v) {
+  __syncwarp();
   v = warp_sum(v);
   if ((threadIdx.x & 31u) == 0) add_counter(c, v);
 }
