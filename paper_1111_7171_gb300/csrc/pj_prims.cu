@@ -176,16 +176,19 @@ __global__ void k_widen(const uint32_t* __restrict__ in, uint64_t* __restrict__ 
   if (i < n) out[i] = in[i];
 }
 
-// The digits of a sort's passes: pass p takes 8 bits from shift[p] (digits
-// that are the same in every key are left out by the caller).
+// The digits of a sort's passes: pass p takes mask[p], at most 8 bits wide,
+// from shift[p] (digits that are the same in every key are left out by the
+// caller).  The mask cuts the last digit to the bits that are sorted by: keys
+// may carry other things above them (the packed accepted matches).
 struct Digits {
   int n;
   int shift[8];
+  unsigned mask[8];
 };
 
 template <class K>
-__device__ __forceinline__ unsigned digit_of(K key, int shift) {
-  return (unsigned)(key >> shift) & 0xFFu;
+__device__ __forceinline__ unsigned digit_of(K key, int shift, unsigned mask) {
+  return (unsigned)(key >> shift) & mask;
 }
 
 // Counts of every pass's digits: hist[pass * 256 + digit] (zero before).
@@ -202,7 +205,7 @@ __global__ void __launch_bounds__(256) k_rs_hist(const K* __restrict__ keys, siz
     const K key = keys[i];
 #pragma unroll
     for (int p = 0; p < 8; ++p)
-      if (p < dg.n) atomicAdd(&h[p * 256 + digit_of(key, dg.shift[p])], 1u);
+      if (p < dg.n) atomicAdd(&h[p * 256 + digit_of(key, dg.shift[p], dg.mask[p])], 1u);
   }
   __syncthreads();
   for (int k = threadIdx.x; k < dg.n * 256; k += 256)
@@ -265,7 +268,7 @@ template <class K, bool VALS>
 __global__ void __launch_bounds__(RS_THREADS, 3) k_rs_pass(const K* __restrict__ kin,
                                                            const uint32_t* __restrict__ vin, K* __restrict__ kout,
                                                            uint32_t* __restrict__ vout, size_t n, int shift,
-                                                           const uint32_t* __restrict__ hist,
+                                                           unsigned mask, const uint32_t* __restrict__ hist,
                                                            unsigned long long* __restrict__ status,
                                                            const unsigned long long* __restrict__ n_dev) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -289,7 +292,7 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_rs_pass(const K* __restrict__
   for (int r = 0; r < RS_ROUNDS; ++r) key[r] = wbase + r * 32 < items ? kin[wbase + r * 32] : ~K(0);
   __syncthreads();
   uint32_t rank[RS_ROUNDS];
-  warp_ranks(wcnt + warp * 256, [&](int r) { return digit_of(key[r], shift); }, rank);
+  warp_ranks(wcnt + warp * 256, [&](int r) { return digit_of(key[r], shift, mask); }, rank);
   __syncthreads();
   // one thread per digit
   const int d = tid;
@@ -324,7 +327,7 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_rs_pass(const K* __restrict__
           unsigned c = 0;
           const K* in = kin - (size_t)((int)tile - (hi - k)) * RS_TILE;
 #pragma unroll 1
-          for (unsigned i = 0; i < RS_TILE; ++i) c += digit_of(in[i], shift) == (unsigned)d;
+          for (unsigned i = 0; i < RS_TILE; ++i) c += digit_of(in[i], shift, mask) == (unsigned)d;
           s[k] = LB_SUM | c;
         }
         before += s[k] & LB_VALUE;
@@ -338,7 +341,7 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_rs_pass(const K* __restrict__
   __syncthreads();
 #pragma unroll
   for (int r = 0; r < RS_ROUNDS; ++r) {
-    const unsigned k = digit_of(key[r], shift);
+    const unsigned k = digit_of(key[r], shift, mask);
     rank[r] += local_start[k] + wcnt[warp * 256 + k];
     stage[rank[r]] = key[r];
   }
@@ -349,7 +352,7 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_rs_pass(const K* __restrict__
     const int j = r * RS_THREADS + tid;
     if (j < items) {
       const K k = stage[j];
-      const uint32_t pos = out_start[digit_of(k, shift)] + (uint32_t)j;
+      const uint32_t pos = out_start[digit_of(k, shift, mask)] + (uint32_t)j;
       kout[pos] = k;
       if (VALS) to[r] = pos;
     }
@@ -401,10 +404,11 @@ __global__ void __launch_bounds__(RSS_THREADS) k_rs_small(K* __restrict__ keys, 
   }
   for (int p = 0; p < dg.n; ++p) {
     const int shift = dg.shift[p];
+    const unsigned mask = dg.mask[p];
     for (int k = tid; k < RSS_WARPS * 256; k += RSS_THREADS) wcnt[k] = 0;
     __syncthreads();
     uint32_t rank[ROUNDS];
-    warp_ranks(wcnt + warp * 256, [&](int r) { return digit_of(key[r], shift); }, rank);
+    warp_ranks(wcnt + warp * 256, [&](int r) { return digit_of(key[r], shift, mask); }, rank);
     __syncthreads();
     uint32_t cnt = 0, incl = 0;
     if (tid < 256) {
@@ -427,7 +431,7 @@ __global__ void __launch_bounds__(RSS_THREADS) k_rs_small(K* __restrict__ keys, 
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < ROUNDS; ++r) {
-      const unsigned d = digit_of(key[r], shift);
+      const unsigned d = digit_of(key[r], shift, mask);
       const uint32_t at = start[d] + wcnt[warp * 256 + d] + rank[r];
       sk[at] = key[r];
       if (VALS) sv[at] = val[r];
@@ -458,7 +462,8 @@ Digits digits_of(unsigned long long bits) {
       continue;
     }
     if (dg.n == 8) fail(PJ_EINVAL, "radix sort: more than 8 digits");
-    dg.shift[dg.n++] = s;
+    dg.shift[dg.n] = s;
+    dg.mask[dg.n++] = (unsigned)(bits >> s) & 0xFFu;
     s += 8;
   }
   return dg;
@@ -537,10 +542,10 @@ bool radix_sort_bits_dn(const Ctx& c, K* keys, uint32_t* vals, K* keys2, uint32_
   for (int p = 0; p < dg.n; ++p) {
     unsigned long long* status = work.p + RS_HIST_WORDS + per_pass * p;
     if (vals)
-      k_rs_pass<K, true><<<ntiles, RS_THREADS, bytes, c.stream>>>(ka, va, kb, vb, cap, dg.shift[p], hist + 256 * p, status,
-                                                              n_dev);
+      k_rs_pass<K, true><<<ntiles, RS_THREADS, bytes, c.stream>>>(ka, va, kb, vb, cap, dg.shift[p], dg.mask[p],
+                                                              hist + 256 * p, status, n_dev);
     else
-      k_rs_pass<K, false><<<ntiles, RS_THREADS, bytes, c.stream>>>(ka, nullptr, kb, nullptr, cap, dg.shift[p],
+      k_rs_pass<K, false><<<ntiles, RS_THREADS, bytes, c.stream>>>(ka, nullptr, kb, nullptr, cap, dg.shift[p], dg.mask[p],
                                                                hist + 256 * p, status, n_dev);
     PJ_LAUNCHED("k_rs_pass");
     K* tk = ka; ka = kb; kb = tk;

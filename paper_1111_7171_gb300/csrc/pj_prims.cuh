@@ -23,9 +23,9 @@ void exclusive_scan(const Ctx& c, const T* in, T* out, size_t n);
 template <class K>
 void radix_sort_pairs(const Ctx& c, K* keys, uint32_t* vals, size_t n, int nbits);
 
-// The same by the set bits of `bits`, which has every bit in which two keys
-// may differ (digits start at set bits; bits that are equal in all keys cost
-// no pass).
+// The same by the set bits of `bits` (digits of up to 8 bits start at set
+// bits, so stretches of clear bits cost no pass).  Here and above, other bits
+// of the key order nothing.
 template <class K>
 void radix_sort_bits(const Ctx& c, K* keys, uint32_t* vals, size_t n, unsigned long long bits);
 
