@@ -134,6 +134,18 @@ struct DBuf {
     n = count;
     p = static_cast<T*>(c.get((count ? count : 1) * sizeof(T)));
   }
+  // The same for a buffer that the work can do without: false, and empty,
+  // when the memory for it cannot be had.
+  bool try_reset(const Ctx& c, size_t count) {
+    try {
+      reset(c, count);
+    } catch (const Error& e) {
+      release();
+      if (e.code != PJ_ENOMEM) throw;
+      return false;
+    }
+    return true;
+  }
   void release() {
     if (p) ctx.put(p);
     p = nullptr;

@@ -635,14 +635,13 @@ void build_store(pj_index& idx, const pj_strings& S) {
                                                                                 idx.sref.p);
     PJ_LAUNCHED("k_refs");
   }
-  // Bit planes for short strings, 32 bytes each (not under a device budget:
-  // they are only for speed).
+  // Bit planes for short strings, 32 bytes each (not under a device budget or
+  // without memory for them: they are only for speed).
   DBuf<uint32_t> bits;
-  const bool planes = n && !c.budget && total <= PLANES_MAX_AVG_LEN * n;
+  const bool planes = n && !c.budget && total <= PLANES_MAX_AVG_LEN * n && idx.splanes.try_reset(c, n);
   if (planes) {
     bits.reset(c, 2);
     PJ_CUDA(cudaMemsetAsync(bits.p, 0, 2 * sizeof(uint32_t), c.stream));
-    idx.splanes.reset(c, n);
     k_byte_bits<<<std::min<unsigned>(ceil_div(total ? total : 1, 256 * 16), sm_grid_cap(8)), 256, 0, c.stream>>>(
         idx.sbytes.p, total, bits.p);
     PJ_LAUNCHED("k_byte_bits");
@@ -944,10 +943,7 @@ void upload_probe_set(const Ctx& c, const pj_index& idx, const pj_strings& R, Pr
   }
   out.bytes = dbytes;
   out.off = doff;
-  if (planes && idx.splanes.p && R.n) {
-    out.planes.reset(c, R.n);
-    query_planes(c, idx, out, out.planes.p);
-  }
+  if (planes && idx.splanes.p && R.n && out.planes.try_reset(c, R.n)) query_planes(c, idx, out, out.planes.p);
   out.own_bytes = std::move(bb);
   out.own_off = std::move(ob);
 }

@@ -1634,6 +1634,15 @@ struct HitTiles {
   DBuf<uint2> list;
   DBuf<uint32_t> rest;
   DBuf<TileCounts> counts;
+  void release() {
+    n_tiles = 0;
+    hits.release();
+    tiles.release();
+    totals.release();
+    list.release();
+    rest.release();
+    counts.release();
+  }
 };
 
 // List entries of one tile range (2 GiB), and listed entries without planes.
@@ -1864,9 +1873,9 @@ struct AcceptBuf {
   }
 };
 
-// Groups n hits over the postings [0, n_postings) of v's index.
-static void group_hits(const Ctx& c, const ProbeView& v, DBuf<Hit>& hits, unsigned long long n,
-                                     HitTiles& t) {
+// Groups n hits over the postings [0, n_postings) of v's index; they move to
+// t.hits.  (An exception leaves them where they are.)
+static void group_hits(const Ctx& c, const ProbeView& v, DBuf<Hit>& hits, unsigned long long n, HitTiles& t) {
   const unsigned long long np = v.n_postings;
   DBuf<uint32_t> cnt(c, 2 * np), off(c, np), rank(c, n);
   uint32_t* longest = cnt.p + np;
@@ -1891,9 +1900,28 @@ static void group_hits(const Ctx& c, const ProbeView& v, DBuf<Hit>& hits, unsign
   hits.release();
 }
 
-// Probe + verify for all probing strings, in chunks of probing strings whose
-// groups fit the hit buffer; then the short-string fallback.  Returns the
-// number of accepted matches (the buffer holds min(that, out.cap)).
+// Candidates per hit and their offsets (n_hits + 1 entries each).
+static void hit_offsets(const Ctx& c, const DBuf<Hit>& hits, unsigned long long n_hits, DBuf<unsigned long long>& cnt,
+                        DBuf<unsigned long long>& off) {
+  cnt.reset(c, n_hits + 1);
+  off.reset(c, n_hits + 1);
+  PJ_CUDA(cudaMemsetAsync(cnt.p + n_hits, 0, sizeof(unsigned long long), c.stream));
+  k_hit_counts<<<ceil_div(n_hits, 256), 256, 0, c.stream>>>(hits.p, n_hits, cnt.p, nullptr);
+  PJ_LAUNCHED("k_hit_counts");
+  exclusive_scan<unsigned long long>(c, cnt.p, off.p, n_hits + 1);
+}
+
+// The queued form for hits that were, or were to be, verified by tiles, when
+// the tiles' buffers do not fit the device: the queued kernel takes the hits
+// in any order.
+static void drop_tiles(const Ctx& c, DBuf<Hit>& hits, unsigned long long n_hits, DBuf<unsigned long long>& cnt,
+                       DBuf<unsigned long long>& off, HitTiles& t) {
+  if (!hits.p) hits = std::move(t.hits);
+  t.release();
+  hit_offsets(c, hits, n_hits, cnt, off);
+  trace_note("join: no memory for tiles");
+}
+
 // Probe one chunk of probing strings: per-group hit counts, their prefix
 // sum, the hits, and the candidate offsets of the hits (n_hits + 1 entries).
 template <bool SELF, bool MULTI>
@@ -1901,7 +1929,7 @@ static void probe_chunk(const Ctx& c, const ProbeView& v, unsigned long long n_g
                         DBuf<uint32_t>& gcount, DBuf<uint32_t>& goff, DBuf<Hit>& hits, DBuf<unsigned long long>& cnt,
                         DBuf<unsigned long long>& off, unsigned long long& n_hits, unsigned long long& n_cand,
                         HitTiles* tiles = nullptr) {
-  if (tiles) tiles->n_tiles = 0;
+  if (tiles) tiles->release();
   gcount.reset(c, n_groups);
   goff.reset(c, n_groups);
   DBuf<unsigned long long> gmask(c, n_groups);
@@ -1922,20 +1950,20 @@ static void probe_chunk(const Ctx& c, const ProbeView& v, unsigned long long n_g
                                                         n_hits);
   PJ_LAUNCHED("k_group_hits");
   trace_mark(c, "join: probe (hits)");
-  cnt.reset(c, n_hits + 1);
-  off.reset(c, n_hits + 1);
-  PJ_CUDA(cudaMemsetAsync(cnt.p + n_hits, 0, sizeof(unsigned long long), c.stream));
-  k_hit_counts<<<ceil_div(n_hits, 256), 256, 0, c.stream>>>(hits.p, n_hits, cnt.p, nullptr);
-  PJ_LAUNCHED("k_hit_counts");
-  exclusive_scan<unsigned long long>(c, cnt.p, off.p, n_hits + 1);
+  hit_offsets(c, hits, n_hits, cnt, off);
   PJ_CUDA(cudaMemcpyAsync(&n_cand, off.p + n_hits, sizeof(n_cand), cudaMemcpyDeviceToHost, c.stream));
   c.sync();
   const unsigned long long knob = env_knob("PJ_TILES_MIN_HITS", 0);
   if (tiles && (knob ? n_hits >= knob : n_hits >= TILES_MIN_HITS && n_cand >= TILES_MIN_RUN * n_hits)) {
     cnt.release();
     off.release();
-    group_hits(c, v, hits, n_hits, *tiles);
-    trace_mark(c, "join: group hits by run");
+    try {
+      group_hits(c, v, hits, n_hits, *tiles);
+      trace_mark(c, "join: group hits by run");
+    } catch (const Error& e) {
+      if (e.code != PJ_ENOMEM) throw;
+      drop_tiles(c, hits, n_hits, cnt, off, *tiles);
+    }
   }
 }
 
@@ -2211,6 +2239,8 @@ static void launch_query(const Ctx& c, const ProbeView& v, unsigned long long n_
   PJ_LAUNCHED("k_query_tasks");
 }
 
+// Probe + verify for all probing strings, in chunks of probing strings whose
+// groups fit the hit buffer; then the short-string fallback.
 template <bool SELF, bool MULTI>
 static void probe_and_verify(const Ctx& c, const ProbeView& v0, uint32_t fb_count, AcceptBuf& acc, Counters* ctr,
                              Counters& h, Timings& tm, const unsigned long long* h_qgoff) {
@@ -2246,12 +2276,13 @@ static void probe_and_verify(const Ctx& c, const ProbeView& v0, uint32_t fb_coun
   if constexpr (!SELF) {  // a query batch: everything up to the accepted matches in one launch
     const unsigned long long groups = MULTI ? h_qgoff[v0.pbegin + v0.pcount] : (unsigned long long)v0.pcount * G;
     if (v0.queued && !v0.pair_mode && groups && groups <= std::min(QUERY_FUSED_MAX_GROUPS, group_budget)) {
-      DBuf<Hit> tasks(c, c.budget ? 1 : QUERY_TASKS);
+      DBuf<Hit> tasks;  // without room, long runs stay with their warps
+      const unsigned long long task_cap = !c.budget && tasks.try_reset(c, QUERY_TASKS) ? QUERY_TASKS : 0;
       tv.start();
       acc.fresh = true;  // nothing has run before it
       acc.run(
           [&](AccOut o) {
-#define PJ_CALL(W) launch_query<W, MULTI>(c, v0, groups, nullptr, tasks.p, c.budget ? 0 : QUERY_TASKS, o, ctr)
+#define PJ_CALL(W) launch_query<W, MULTI>(c, v0, groups, nullptr, tasks.p, task_cap, o, ctr)
             PJ_BY_TAU(v0.tau, PJ_CALL);
 #undef PJ_CALL
           },
@@ -2312,53 +2343,69 @@ static void probe_and_verify(const Ctx& c, const ProbeView& v0, uint32_t fb_coun
       // The list holds a quarter of the candidates (about 9% survive on short
       // strings at tau = 4), at most LIST_MAX; a range whose survivors do not
       // fit is screened again in halves.  Accepted matches never exceed the
-      // list, so the verification never runs twice.
+      // list, so the verification never runs twice.  Without memory for the
+      // list or for the survivors among the accepted matches, what the chunk
+      // has counted and accepted is taken back and the queued form runs.
       const unsigned long long T = tiles.n_tiles;
-      const unsigned long long want =
-          std::min({n_cand + (1ull << 20), std::max(n_cand / 4, 1ull << 22), LIST_MAX, env_knob("PJ_LAUNCH_CANDS", LIST_MAX)});
-      if (tiles.list.n < want) tiles.list.reset(c, want);
-      if (!tiles.rest.p) tiles.rest.reset(c, REST_MAX);
-      if (!tiles.counts.p) tiles.counts.reset(c, 1);
-      tv.start();
-      double share = (double)tiles.list.n / (0.2 * (double)n_cand);  // of the tiles whose survivors fit, expected
-      for (unsigned long long tb = 0; tb < T;) {
-        const unsigned long long step =
-            std::max<unsigned long long>(1, (unsigned long long)(std::min(1.0, share) * (double)T));
-        const unsigned long long te = std::min(T, tb + step);
-        Counters saved{};
-        PJ_CUDA(cudaMemcpyAsync(&saved, ctr, sizeof(saved), cudaMemcpyDeviceToHost, c.stream));
-        const unsigned long long n = screen_tiles(c, v, tiles, tb, te, ctr);
-        if (n > tiles.list.n) {
-          PJ_CUDA(cudaMemcpyAsync(ctr, &saved, sizeof(saved), cudaMemcpyHostToDevice, c.stream));
-          c.sync();
-          if (step == 1) {  // one tile's survivors (at most TILE_POSTS * TILE_HITS and a chunk)
-            tiles.list.reset(c, (unsigned long long)TILE_POSTS * TILE_HITS + 8 * T_FLUSH);
-          } else {
-            share = 0.5 * (double)step / (double)T;
+      Counters before{};
+      bool counted = false;
+      try {
+        const unsigned long long want = std::min(
+            {n_cand + (1ull << 20), std::max(n_cand / 4, 1ull << 22), LIST_MAX, env_knob("PJ_LAUNCH_CANDS", LIST_MAX)});
+        tiles.list.reset(c, want);
+        tiles.rest.reset(c, REST_MAX);
+        tiles.counts.reset(c, 1);
+        tv.start();
+        double share = (double)tiles.list.n / (0.2 * (double)n_cand);  // of the tiles whose survivors fit, expected
+        for (unsigned long long tb = 0; tb < T;) {
+          const unsigned long long step =
+              std::max<unsigned long long>(1, (unsigned long long)(std::min(1.0, share) * (double)T));
+          const unsigned long long te = std::min(T, tb + step);
+          Counters saved{};
+          PJ_CUDA(cudaMemcpyAsync(&saved, ctr, sizeof(saved), cudaMemcpyDeviceToHost, c.stream));
+          const unsigned long long n = screen_tiles(c, v, tiles, tb, te, ctr);
+          if (!counted) before = saved;
+          counted = true;
+          if (n > tiles.list.n) {
+            PJ_CUDA(cudaMemcpyAsync(ctr, &saved, sizeof(saved), cudaMemcpyHostToDevice, c.stream));
+            c.sync();
+            if (step == 1) {  // one tile's survivors (at most TILE_POSTS * TILE_HITS and a chunk)
+              tiles.list.reset(c, (unsigned long long)TILE_POSTS * TILE_HITS + 8 * T_FLUSH);
+            } else {
+              share = 0.5 * (double)step / (double)T;
+            }
+            continue;
           }
-          continue;
-        }
-        share = std::min(2.0 * (double)step / (double)T, 0.9 * (double)tiles.list.n / (double)std::max(1ull, n) *
-                                                             ((double)(te - tb) / (double)T));
-        if (n) {
-          if (acc.last + n > acc.cap) acc.reserve(std::max(acc.last + n, acc.cap + acc.cap / 2));
-          acc.run(
-              [&](AccOut o) {
+          share = std::min(2.0 * (double)step / (double)T, 0.9 * (double)tiles.list.n / (double)std::max(1ull, n) *
+                                                               ((double)(te - tb) / (double)T));
+          if (n) {
+            if (acc.last + n > acc.cap) acc.reserve(std::max(acc.last + n, acc.cap + acc.cap / 2));
+            acc.run(
+                [&](AccOut o) {
 #define PJ_CALL(W) launch_list<W, SELF>(c, v, tiles, n, o, ctr)
-                PJ_BY_TAU(v.tau, PJ_CALL);
+                  PJ_BY_TAU(v.tau, PJ_CALL);
 #undef PJ_CALL
-              },
-              [&](unsigned long long after) { return 2 * after; });
+                },
+                [&](unsigned long long after) { return 2 * after; });
+          }
+          tb = te;
         }
-        tb = te;
+        tv.stop();
+        tm.verify += tv.ms();
+        verified += n_cand;
+        tile_cand += n_cand;
+        trace_mark(c, "join: verify (tiles)");
+        done += v.pcount;
+        continue;
+      } catch (const Error& e) {
+        if (e.code != PJ_ENOMEM) throw;
       }
-      tv.stop();
-      tm.verify += tv.ms();
-      verified += n_cand;
-      tile_cand += n_cand;
-      trace_mark(c, "join: verify (tiles)");
-      done += v.pcount;
-      continue;
+      if (counted) {
+        PJ_CUDA(cudaMemcpyAsync(ctr, &before, sizeof(before), cudaMemcpyHostToDevice, c.stream));
+        c.sync();  // `before` lives on this stack frame
+        acc.last = before.accepted;
+      }
+      drop_tiles(c, hits, n_hits, cnt, off, tiles);
     }
     // Joins of up to SIZING_MIN_CANDS candidates verify in one launch with
     // room for 1/16 of them accepted; bigger ones first verify 1/64 of their

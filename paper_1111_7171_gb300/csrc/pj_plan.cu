@@ -227,12 +227,12 @@ void create(pj_plan& P, pj_index& idx, const pj_plan_options& o) {
   P.sizes.reset(P.ctx, 1);
   P.len.reset(P.ctx, d.cap_q);
   P.bm.reset(P.ctx, d.cap_q);
-  if (idx.splanes.p) P.planes.reset(P.ctx, d.cap_q);
+  if (idx.splanes.p) P.planes.try_reset(P.ctx, d.cap_q);  // without them, matches are verified on the bytes
   P.gcnt.reset(P.ctx, d.cap_q);
   P.qgoff.reset(P.ctx, d.cap_q);
   P.counters.reset(P.ctx, PLAN_COUNTER_BYTES);
   d.task_cap = std::min<uint64_t>(1u << 18, std::max<uint64_t>(1u << 12, cap_groups));
-  P.tasks.reset(P.ctx, d.task_cap);
+  if (!P.tasks.try_reset(P.ctx, d.task_cap)) d.task_cap = 0;  // long runs then stay with their warps
   d.tasks = P.tasks.p;
   d.bytes = P.bytes.p;
   d.off = P.off.p;
