@@ -957,7 +957,7 @@ uint64_t pj_index::device_bytes() const {
                sref.bytes() + splanes.bytes();
   for (const auto& p : parts)
     b += p.table.bytes() + p.fp.bytes() + p.postings.bytes() + p.precs.bytes() + p.gorder[0].bytes() +
-         p.gorder[1].bytes();
+         p.gorder[1].bytes() + p.pmask.bytes();
   return b;
 }
 
