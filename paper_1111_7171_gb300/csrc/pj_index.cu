@@ -439,13 +439,12 @@ __global__ void k_table_insert(const unsigned long long* __restrict__ keys, cons
 }
 
 // The bitmap behind the position masks: (value, segment length) of every
-// distinct key, two bits of one word as in the presence bitmap.
-__global__ void k_value_bits(const unsigned long long* __restrict__ keys, const uint32_t* __restrict__ heads,
-                             uint64_t n_unique, int tau, int scheme, unsigned long long magic, unsigned pb,
-                             unsigned long long mask, uint32_t* __restrict__ bitmap) {
-  const uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (u >= n_unique) return;
-  const unsigned long long key = keys[heads[u]];
+// key of the table, two bits of one word as in the presence bitmap.
+__global__ void k_value_bits(const Slot* __restrict__ table, int tau, int scheme, unsigned long long magic,
+                             unsigned pb, unsigned long long mask, uint32_t* __restrict__ bitmap) {
+  const uint64_t h = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned long long key = h <= mask ? table[h].key : 0ull;
+  if (key == 0) return;
   int P, li;
   segment_m((int)((key >> 8) & 0xFFFFFFu), tau + 1, magic, scheme, (int)(key & 0xFFu), P, li);
   if (li <= SEG_EXACT_MAX) return;
@@ -693,35 +692,36 @@ static uint64_t window_positions(int tau) {
 // Position masks (k_position_masks) for indexes of long strings, when the
 // windows select a position at least MASKS_MIN_SHARE times for every test that
 // the masks make of it (3 per byte).  Under a device budget, or without
-// memory for them, the join looks every position up.
+// memory for them, the join looks every position up.  Only self joins read
+// them, so R x S joins and indexes that answer queries never pay for them (1.1
+// ms and 0.375 bytes a byte at 100k strings of 1,000).
 constexpr uint64_t MASKS_MIN_SHARE = 2;
 
-static void build_position_masks(const pj_index& idx, Partition& part, const unsigned long long* keys,
-                                 const uint32_t* heads) {
+void ensure_position_masks(const pj_index& idx, Partition& part, float* ms) {
   const Ctx& c = idx.ctx;
-  if (part.sides || c.budget || !idx.sph.p) return;
+  if (part.pmask_asked) return;
+  part.pmask_asked = true;
+  if (part.n_records == 0 || part.sides || c.budget || !idx.sph.p) return;
   if (window_positions(part.tau) * idx.n < MASKS_MIN_SHARE * 3 * idx.total_bytes) return;
   const uint64_t cap = part.table.n;
   DBuf<uint32_t> bitmap;
-  try {
-    bitmap.reset(c, cap * part.presence_bytes / 4);
-    part.pmask.reset(c, 3 * (mask_word(idx.total_bytes, idx.n) + 1));
-  } catch (const Error& e) {
-    if (e.code != PJ_ENOMEM) throw;
-    bitmap.release();
-    part.pmask.release();
+  if (!bitmap.try_reset(c, cap * part.presence_bytes / 4) ||
+      !part.pmask.try_reset(c, 3 * (mask_word(idx.total_bytes, idx.n) + 1)))
     return;
-  }
+  EventTimer t(c.stream);
+  t.start();
   PJ_CUDA(cudaMemsetAsync(bitmap.p, 0, bitmap.bytes(), c.stream));
-  k_value_bits<<<ceil_div(part.n_unique, 256), 256, 0, c.stream>>>(keys, heads, part.n_unique, part.tau, part.scheme,
-                                                                   seg_magic(part.tau + 1), part.presence_bytes,
-                                                                   cap - 1, bitmap.p);
+  k_value_bits<<<ceil_div(cap, 256), 256, 0, c.stream>>>(part.table.p, part.tau, part.scheme, seg_magic(part.tau + 1),
+                                                         part.presence_bytes, cap - 1, bitmap.p);
   PJ_LAUNCHED("k_value_bits");
   const uint32_t np = idx.n - part.first;
   k_position_masks<<<std::min<unsigned>(ceil_div(np, 8), sm_grid_cap(8)), 256, 0, c.stream>>>(
       idx.soff.p, idx.slen.p, idx.sph.p, part.first, idx.n, part.tau, part.presence_bytes, cap - 1, bitmap.p,
       part.pmask.p);
   PJ_LAUNCHED("k_position_masks");
+  t.stop();
+  if (ms) *ms += t.ms();
+  trace_mark(c, "partition: position masks");
 }
 
 // Window size of group (length offset, segment i) when nothing clips it
@@ -830,7 +830,6 @@ void build_partition(pj_index& idx, int tau, Partition& part) {
         part.postings.p, keys.p, nrec, part.first, tau, sides.p, part.precs.p);
     PJ_LAUNCHED("k_post_records");
   }
-  build_position_masks(idx, part, keys.p, heads.p);
   trace_mark(c, "partition: table");
   if (getenv("PJ_CHECK_INDEX")) check_partition(c, part);
   if (getenv("PJ_DEBUG_DUMP")) {

@@ -601,8 +601,10 @@ struct Partition {
   // by window size, widest first; [0] for R != S probes, [1] for the self join
   DBuf<uint16_t> gorder[2];
   // position masks of the indexed strings as probes of the self join
-  // (k_position_masks; empty: not built)
+  // (k_position_masks; empty: not built), and whether a self join has asked
+  // for them
   DBuf<uint32_t> pmask;
+  bool pmask_asked = false;
 };
 
 }  // namespace pj
@@ -650,6 +652,9 @@ void build_partition(pj_index& idx, int tau, Partition& part);
 // Returns idx.parts[tau], building it first if the index is lazy and it is
 // not built yet (*ms receives the device time spent, else 0).
 Partition& ensure_partition(pj_index& idx, int tau, float* ms);
+// Builds part's position masks where they pay, when a self join first asks
+// for them; adds the device time to *ms.
+void ensure_position_masks(const pj_index& idx, Partition& part, float* ms);
 
 // Device copy of a probe set (R or a query batch) in input order.
 struct ProbeSet {

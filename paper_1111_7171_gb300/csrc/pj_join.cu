@@ -3468,6 +3468,7 @@ static void self_join_impl(pj_index& idx, int tau, pj_result* out, bool on_devic
   const bool whole = q_lo == 0 && q_hi >= idx.n && fallback != 0;
   float part_ms = 0.f;
   ensure_partition(idx, tau, &part_ms);
+  ensure_position_masks(idx, idx.parts[tau], &part_ms);
   struct DumpAfter {
     pj_index& idx;
     int tau;

@@ -24,3 +24,16 @@ def test_masks_are_counted():
     assert idx.device_bytes - without.device_bytes == masks
     idx.free()
     without.free()
+
+
+def test_masks_wait_for_a_self_join():
+    """Only self joins read masks: building, queries and R x S joins make none."""
+    strings, masks, (idx, without) = indexes()
+    for i in (idx, without):
+        assert len(pj.pj_query(i, strings[:3], TAU).pairs) >= 3  # builds the threshold
+    assert idx.device_bytes == without.device_bytes
+    first = [pj.pj_self_join(i, TAU).pairs for i in (idx, without)]
+    assert len(first[0]) and (first[0] == first[1]).all()
+    assert idx.device_bytes - without.device_bytes == masks
+    idx.free()
+    without.free()
