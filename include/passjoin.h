@@ -166,11 +166,13 @@ typedef struct {
                              later self joins of the threshold replay it (one graph launch;
                              same results; a count above a recorded capacity, which an
                              unchanged index cannot produce, falls back to the eager path).
-                             Not recorded: joins with a warp-per-candidate range, or with more
+                             Not recorded: joins with a warp-per-candidate range, with more
                              probe groups than PJ_GRAPH_MAX_GROUPS (environment, default
-                             2^28; the graph probes all groups in one pass).  A recorded join
-                             keeps its device buffers (about the eager join's peak scratch;
-                             ~10 GB for 1M short strings at tau = 4) until pj_index_free. */
+                             2^28; the graph probes all groups in one pass), or whose hits
+                             are grouped by posting run, as those of large sets of short
+                             strings are (faster than the recorded form).  A recorded join
+                             keeps its device buffers (about the eager join's peak scratch)
+                             until pj_index_free. */
   uint64_t device_budget; /* 0 = no limit.  Most device memory held at once through this
                              index's allocator (pj_build_index: its store, every threshold's
                              segment index, the scratch of every join, device results) or

@@ -1808,6 +1808,7 @@ static unsigned long long env_knob(const char* name, unsigned long long dflt) {
 struct Timings {
   float probe = 0.f, verify = 0.f, fallback = 0.f, dedupe = 0.f;
   unsigned long long distinct = 0;  // mode L: distinct pairs verified
+  bool tiled = false;               // candidates were verified by tiles
 };
 
 // Accepted-match buffer that grows between launches: after a launch that
@@ -2394,6 +2395,7 @@ static void probe_and_verify(const Ctx& c, const ProbeView& v0, uint32_t fb_coun
         tm.verify += tv.ms();
         verified += n_cand;
         tile_cand += n_cand;
+        tm.tiled = true;
         trace_mark(c, "join: verify (tiles)");
         done += v.pcount;
         continue;
@@ -2491,8 +2493,9 @@ static void probe_and_verify(const Ctx& c, const ProbeView& v0, uint32_t fb_coun
 }
 
 // Runs the join, retries once with an exact-size buffer if the accepted
-// matches overflowed, then dedupes and compacts into *out.
-static void run_join(const Ctx& c, const ProbeView& v, bool self, uint32_t fb_count, int a_bits,
+// matches overflowed, then dedupes and compacts into *out.  True when
+// candidates were verified by tiles.
+static bool run_join(const Ctx& c, const ProbeView& v, bool self, uint32_t fb_count, int a_bits,
                      bool results_on_device, pj_result* out, const unsigned long long* h_qgoff = nullptr) {
   Counters h{};
   Timings tm;
@@ -2621,6 +2624,7 @@ static void run_join(const Ctx& c, const ProbeView& v, bool self, uint32_t fb_co
     c.sync();
     trace_mark(c, "join: results to host");
   }
+  return tm.tiled;
 }
 
 // ------------------------------------------------------------ autotune ----
@@ -3007,7 +3011,12 @@ static ProbeView index_side(const pj_index& idx, const Partition& part) {
 // (which an unchanged index cannot produce) is discarded and the join runs
 // eagerly.  Not recorded: joins with a warp-per-candidate range, or with more
 // than PJ_GRAPH_MAX_GROUPS probe groups (2^28 by default; the graph probes
-// all groups in one pass, where the eager join takes chunks).
+// all groups in one pass, where the eager join takes chunks), or that verified
+// candidates by tiles: the graph has the queued kernel, which is slower there
+// by more than the launches it saves.  Replay / eager join by tiles, short
+// strings: 100k, tau 4 2.28 / 2.08 ms; 417k, tau 3 5.4 / 4.4; 1M, tau 3 25.0 /
+// 16.4; 1M, tau 4 144 / 103; and without tiles 60k, tau 4 1.12 / 1.24, 1M, tau 2
+// 3.06 / 3.21.
 
 // fz (the fused form, else NULL): fz[2] nonzero when one of its lists
 // outgrew its capacity; its candidates are then counted in ctr->candidates.
@@ -3542,8 +3551,8 @@ static void self_join_impl(pj_index& idx, int tau, pj_result* out, bool on_devic
       idx.self_plans[tau].reset();
     }
   }
-  run_join(idx.ctx, v, true, fb_count, bits_for(idx.n), on_device, out);
-  if (idx.graph_joins && whole && !idx.self_plans[tau]) {
+  const bool tiled = run_join(idx.ctx, v, true, fb_count, bits_for(idx.n), on_device, out);
+  if (idx.graph_joins && whole && !tiled && !idx.self_plans[tau]) {
     try {  // a join that cannot be recorded (device or host memory) still has its result
       std::shared_ptr<SelfPlan> p = make_self_plan(idx, v, tr, part.first, out->stats, out->count);
       if (p) idx.self_plans[tau] = std::static_pointer_cast<void>(p);

@@ -456,7 +456,8 @@ def pj_build_index(strings, tau_max: int, stream=None, results_on_device: bool =
     lazy_partitions: a threshold's segment index is built on its first use.
     autotune: each threshold's self join picks its verification form by timing.
     graph_joins: after a threshold's first self join, later self joins of it
-    replay that join recorded as one CUDA graph (pj_options.graph_joins).
+    replay that join recorded as one CUDA graph, where that is the faster form
+    (pj_options.graph_joins).
     device_budget: most device bytes the index and its calls may hold at once
     (0 = no limit; beyond it a call fails with PJ_ENOMEM).
     autotune_cache: file keeping autotuning decisions across processes.
