@@ -18,7 +18,10 @@ namespace pj {
 constexpr unsigned long long LB_SUM = 1ull << 62;     // the tile's own sum
 constexpr unsigned long long LB_PREFIX = 2ull << 62;  // the sum of all tiles up to it
 constexpr unsigned long long LB_VALUE = (1ull << 62) - 1;
-constexpr int LB_POLLS = 1 << 12;
+#ifndef PJ_LB_POLLS  // a test compiles with 0: every tile that is not done yet is summed again
+#define PJ_LB_POLLS (1 << 12)
+#endif
+constexpr int LB_POLLS = PJ_LB_POLLS;
 
 __device__ __forceinline__ unsigned long long lb_load(const unsigned long long* p) {
   return *reinterpret_cast<const volatile unsigned long long*>(p);
