@@ -242,13 +242,19 @@ __global__ void k_signatures(const uint8_t* __restrict__ bytes, const uint64_t* 
     bm[k] = char_signature(bytes + off[k], (int)(off[k + 1] - off[k]));
 }
 
-// The same, a warp each.
+// The same, a warp each, and bit planes (planes NULL: none).
 __global__ void k_signatures_warp(const uint8_t* __restrict__ bytes, const uint64_t* __restrict__ off, uint32_t n,
-                                  Sig* __restrict__ bm) {
+                                  Sig* __restrict__ bm, ByteBits bb, Planes* __restrict__ planes) {
   const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   for (uint64_t k = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += n_warps) {
-    const Sig t = warp_signature(bytes + off[k], (int)(off[k + 1] - off[k]));
-    if ((threadIdx.x & 31u) == 0) bm[k] = t;
+    const uint8_t* p = bytes + off[k];
+    const int len = (int)(off[k + 1] - off[k]);
+    const Sig t = warp_signature(p, len);
+    const Planes pl = planes ? warp_planes(p, len, bb) : Planes{};
+    if ((threadIdx.x & 31u) == 0) {
+      bm[k] = t;
+      if (planes) planes[k] = pl;
+    }
   }
 }
 
@@ -514,15 +520,22 @@ __global__ void __launch_bounds__(256) k_position_masks(const uint64_t* __restri
 constexpr uint64_t SIG_WARP_AVG_LEN = 256;
 constexpr uint32_t SIG_WARP_STRINGS = 1u << 15;
 
+// planes (NULL: none): the strings' bit planes for bb, by the same launch in
+// the warps' form.
 static void launch_signatures(const Ctx& c, const uint8_t* bytes, const uint64_t* off, uint32_t n, uint64_t total,
-                              Sig* bm) {
+                              Sig* bm, ByteBits bb = {}, Planes* planes = nullptr) {
   if (n <= SIG_WARP_STRINGS || total > SIG_WARP_AVG_LEN * n) {
-    k_signatures_warp<<<std::min<unsigned>(ceil_div((size_t)n * 32, 256), sm_grid_cap(8)), 256, 0, c.stream>>>(bytes, off,
-                                                                                                              n, bm);
+    k_signatures_warp<<<std::min<unsigned>(ceil_div((size_t)n * 32, 256), sm_grid_cap(8)), 256, 0, c.stream>>>(
+        bytes, off, n, bm, bb, planes);
     PJ_LAUNCHED("k_signatures_warp");
   } else {
     k_signatures<<<std::min<unsigned>(ceil_div(n, 256), sm_grid_cap(8)), 256, 0, c.stream>>>(bytes, off, n, bm);
     PJ_LAUNCHED("k_signatures");
+    if (planes) {
+      k_planes<<<std::min<unsigned>(ceil_div(n, 128), sm_grid_cap(16)), 128, 0, c.stream>>>(bytes, off, n, nullptr, bb,
+                                                                                           planes);
+      PJ_LAUNCHED("k_planes");
+    }
   }
 }
 
@@ -904,13 +917,11 @@ Partition& ensure_partition(pj_index& idx, int tau, float* ms) {
   return part;
 }
 
-void query_planes(const Ctx& c, const pj_index& idx, const ProbeSet& R, Planes* out) {
-  k_planes<<<std::min<unsigned>(ceil_div(R.n, 128), sm_grid_cap(16)), 128, 0, c.stream>>>(R.bytes, R.off, R.n, nullptr,
-                                                                                         idx.byte_bits, out);
-  PJ_LAUNCHED("k_planes");
+void query_signatures(const Ctx& c, const pj_index& idx, ProbeSet& R, Planes* planes) {
+  if (R.n) launch_signatures(c, R.bytes, R.off, R.n, R.total, R.bm.p, idx.byte_bits, planes);
 }
 
-void upload_probe_set(const Ctx& c, const pj_index& idx, const pj_strings& R, ProbeSet& out, bool planes) {
+void upload_probe_set(const Ctx& c, const pj_index& idx, const pj_strings& R, ProbeSet& out, bool signatures) {
   const uint8_t* dbytes = nullptr;
   const uint64_t* doff = nullptr;
   uint64_t total = 0;
@@ -921,28 +932,26 @@ void upload_probe_set(const Ctx& c, const pj_index& idx, const pj_strings& R, Pr
   // keep the device copy (host input) or reference the caller's (device input)
   out.len.reset(c, R.n);
   DBuf<uint32_t> ids(c, R.n);
-  DBuf<int> err(c, 1);
-  DBuf<unsigned> lmax(c, 1);
-  PJ_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), c.stream));
-  PJ_CUDA(cudaMemsetAsync(lmax.p, 0, sizeof(unsigned), c.stream));
+  DBuf<unsigned> found(c, 2);  // an error, the longest length
+  PJ_CUDA(cudaMemsetAsync(found.p, 0, 2 * sizeof(unsigned), c.stream));
   if (R.n) {
-    k_lengths<<<ceil_div(R.n, 256), 256, 0, c.stream>>>(doff, R.n, out.len.p, ids.p, err.p, lmax.p);
+    k_lengths<<<ceil_div(R.n, 256), 256, 0, c.stream>>>(doff, R.n, out.len.p, ids.p, reinterpret_cast<int*>(found.p),
+                                                       found.p + 1);
     PJ_LAUNCHED("k_lengths");
   }
-  int h_err = 0;
-  unsigned h_lmax = 0;
-  PJ_CUDA(cudaMemcpyAsync(&h_err, err.p, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
-  PJ_CUDA(cudaMemcpyAsync(&h_lmax, lmax.p, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream));
+  unsigned h_found[2] = {0, 0};
+  PJ_CUDA(cudaMemcpyAsync(h_found, found.p, sizeof(h_found), cudaMemcpyDeviceToHost, c.stream));
   c.sync();
-  if (h_err) fail(PJ_EINVAL, "pj_strings: offsets decrease or a string is longer than 65535 bytes");
-  out.lmax = (int)h_lmax;
+  if (h_found[0]) fail(PJ_EINVAL, "pj_strings: offsets decrease or a string is longer than 65535 bytes");
+  out.lmax = (int)h_found[1];
   out.bm.reset(c, R.n ? R.n : 1);
-  if (R.n) {
-    launch_signatures(c, dbytes, doff, R.n, total, out.bm.p);
-  }
   out.bytes = dbytes;
   out.off = doff;
-  if (planes && idx.splanes.p && R.n && out.planes.try_reset(c, R.n)) query_planes(c, idx, out, out.planes.p);
+  out.total = total;
+  if (signatures) {
+    if (idx.splanes.p && R.n) out.planes.try_reset(c, R.n);
+    query_signatures(c, idx, out, out.planes.p);
+  }
   out.own_bytes = std::move(bb);
   out.own_off = std::move(ob);
 }

@@ -667,12 +667,13 @@ struct ProbeSet {
   DBuf<Planes> planes;  // bit planes (when the index has them)
   uint32_t n = 0;
   int lmax = 0;
+  uint64_t total = 0;  // bytes
 };
-// planes: with bit planes if idx has them.
-void upload_probe_set(const Ctx& c, const pj_index& idx, const pj_strings& R, ProbeSet& out, bool planes = true);
+// signatures: with their signatures, and bit planes if idx has them.
+void upload_probe_set(const Ctx& c, const pj_index& idx, const pj_strings& R, ProbeSet& out, bool signatures = true);
 
-// Bit planes of R's strings for idx (which has them).
-void query_planes(const Ctx& c, const pj_index& idx, const ProbeSet& R, Planes* out);
+// Signatures of R's strings, and their bit planes for idx (planes NULL: none).
+void query_signatures(const Ctx& c, const pj_index& idx, ProbeSet& R, Planes* planes);
 
 // R != S probe of a resident index where probe q has threshold h_tau[q]
 // (host array).  Every threshold present must be built.  Work is ordered on

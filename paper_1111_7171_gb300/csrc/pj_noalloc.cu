@@ -163,7 +163,7 @@ void query_noalloc(pj_index& idx, const pj_strings& batch, int tau, pj_pair* out
   c.alloc_ctx = &bump;
 
   ProbeSet R;
-  upload_probe_set(c, idx, batch, R, false);  // device input: lengths and signatures only, in the scratch
+  upload_probe_set(c, idx, batch, R, false);  // device input: lengths, and room for signatures, in the scratch
   DBuf<Counters> ctr(c, 1);
   PJ_CUDA(cudaMemsetAsync(ctr.p, 0, sizeof(Counters), c.stream));
 
@@ -183,9 +183,9 @@ void query_noalloc(pj_index& idx, const pj_strings& batch, int tau, pj_pair* out
   size_t spare = (1u << 20) - (1u << 16) + 4 * cap;
   if (idx.splanes.p && R.n && align256((size_t)R.n * sizeof(Planes)) <= spare) {
     planes.reset(c, R.n);
-    query_planes(c, idx, R, planes.p);
     spare -= align256((size_t)R.n * sizeof(Planes));
   }
+  query_signatures(c, idx, R, planes.p);
   if (spare >= (1u << 16)) tasks.reset(c, std::min<size_t>(1u << 16, spare / 2 / sizeof(Hit)));
 
   ProbeView v{};
