@@ -2225,7 +2225,7 @@ static bool fused_self_join(const Ctx& c, const ProbeView& v, AcceptBuf& acc, Co
 // R != S join takes the probe passes, whose lanes roll a window's keys.
 constexpr unsigned long long QUERY_FUSED_MAX_GROUPS = 1ull << 18;
 
-// Room for the parts of a batch's long runs: 8 MiB.
+// Least room for the parts of a batch's long runs (query_task_room): 8 MiB.
 constexpr unsigned long long QUERY_TASKS = 1ull << 18;
 
 template <int MAXW, bool MULTI>
@@ -2278,7 +2278,8 @@ static void probe_and_verify(const Ctx& c, const ProbeView& v0, uint32_t fb_coun
     const unsigned long long groups = MULTI ? h_qgoff[v0.pbegin + v0.pcount] : (unsigned long long)v0.pcount * G;
     if (v0.queued && !v0.pair_mode && groups && groups <= std::min(QUERY_FUSED_MAX_GROUPS, group_budget)) {
       DBuf<Hit> tasks;  // without room, long runs stay with their warps
-      const unsigned long long task_cap = !c.budget && tasks.try_reset(c, QUERY_TASKS) ? QUERY_TASKS : 0;
+      unsigned long long task_cap = c.budget ? 0 : std::max(QUERY_TASKS, query_task_room(groups, v0.n_index));
+      while (task_cap && !tasks.try_reset(c, task_cap)) task_cap = task_cap / 2 >= QUERY_TASKS ? task_cap / 2 : 0;
       tv.start();
       acc.fresh = true;  // nothing has run before it
       acc.run(

@@ -231,8 +231,9 @@ void create(pj_plan& P, pj_index& idx, const pj_plan_options& o) {
   P.gcnt.reset(P.ctx, d.cap_q);
   P.qgoff.reset(P.ctx, d.cap_q);
   P.counters.reset(P.ctx, PLAN_COUNTER_BYTES);
-  d.task_cap = std::min<uint64_t>(1u << 18, std::max<uint64_t>(1u << 12, cap_groups));
-  if (!P.tasks.try_reset(P.ctx, d.task_cap)) d.task_cap = 0;  // long runs then stay with their warps
+  d.task_cap = query_task_room(cap_groups, idx.n);
+  while (d.task_cap && !P.tasks.try_reset(P.ctx, d.task_cap))  // without any, long runs stay with their warps
+    d.task_cap = d.task_cap > (1u << 12) ? d.task_cap / 2 : 0;
   d.tasks = P.tasks.p;
   d.bytes = P.bytes.p;
   d.off = P.off.p;

@@ -122,6 +122,18 @@ inline size_t sort_temp_bytes(size_t n) {
   return align256(8 * (RS_HIST_WORDS + 8 * 256 * ((n + RS_TILE - 1) / RS_TILE)));
 }
 
+// Room for the parts of long runs that a batch of `groups` groups sets aside
+// (k_query_fused, 32 bytes each): 2^12 for small batches, at most 256 MiB.  A
+// million short strings have between 1.4 and 2.7 parts a group at tau <= 4, and
+// the runs grow with the index.  Parts without room are walked where they were
+// found, unevenly: a plan's batch of 16,384 queries of mixed thresholds takes
+// 4.1 ms with room for 2^18 parts and 2.2 ms with room for all, one of 65,536
+// 15.8 and 9.0 ms.
+inline unsigned long long query_task_room(unsigned long long groups, uint32_t n_index) {
+  if (groups <= 1ull << 12) return 1ull << 12;
+  return std::min(1ull << 23, 4 * groups * std::max(1u, n_index >> 20));
+}
+
 // Enqueues the whole query pipeline for the buffers in d on c's stream
 // without any host synchronisation (meant to run under stream capture).
 // Temporaries come from c's allocator and must outlive the recorded work.
