@@ -326,8 +326,8 @@ typedef struct {
 typedef struct {
   uint64_t runs;             /* batches run */
   uint64_t recaptures;       /* graph recordings after the first (capacity growth) */
-  uint32_t graph_nodes;      /* nodes of the current graph */
-  uint32_t graph_kernels;    /* kernel nodes of the current graph (launches per run) */
+  uint32_t graph_nodes;      /* nodes of the graph that the last batch ran (large batches */
+  uint32_t graph_kernels;    /* may have another); its kernel nodes (launches per run) */
   uint64_t hits_capacity, accepted_capacity, pairs_capacity;
   uint64_t device_bytes;     /* device memory held by the plan */
   uint64_t host_bytes;       /* pinned host memory held by the plan */

@@ -2221,10 +2221,6 @@ static bool fused_self_join(const Ctx& c, const ProbeView& v, AcceptBuf& acc, Co
   return true;
 }
 
-// Groups up to which a query batch runs in one launch (k_query_fused); a larger
-// R != S join takes the probe passes, whose lanes roll a window's keys.
-constexpr unsigned long long QUERY_FUSED_MAX_GROUPS = 1ull << 18;
-
 // Least room for the parts of a batch's long runs (query_task_room): 8 MiB.
 constexpr unsigned long long QUERY_TASKS = 1ull << 18;
 
@@ -3694,12 +3690,13 @@ __global__ void k_plan_groups(const uint8_t* __restrict__ bytes, const uint64_t*
   }
 }
 
-__global__ void k_plan_finish(const Counters* __restrict__ ctr, const PlanSizes* __restrict__ sizes,
+// passes: the probe passes counted hits and candidates, else the query kernel.
+__global__ void k_plan_finish(const Counters* __restrict__ ctr, const PlanSizes* __restrict__ sizes, bool passes,
                               PlanHeader* header) {
   PlanHeader h;
   h.groups = sizes->groups;
-  h.hits = ctr->hits;
-  h.cands = ctr->candidates;
+  h.hits = passes ? sizes->hits : ctr->hits;
+  h.cands = passes ? sizes->cands : ctr->candidates;
   h.accepted = ctr->accepted;
   h.pairs = sizes->pairs;
   h.lookups = ctr->lookups;
@@ -3711,7 +3708,7 @@ __global__ void k_plan_finish(const Counters* __restrict__ ctr, const PlanSizes*
   *header = h;
 }
 
-void record_query_plan(const Ctx& c, const pj_index& idx, const PlanDev& d) {
+void record_query_plan(const Ctx& c, const pj_index& idx, const PlanDev& d, bool passes) {
   const int tau_max = (int)idx.parts.size() - 1;
   ProbeView v = index_side(idx, idx.parts[tau_max]);
   v.pbytes = d.bytes;
@@ -3738,11 +3735,32 @@ void record_query_plan(const Ctx& c, const pj_index& idx, const PlanDev& d) {
                                                         idx.byte_bits, d.gcnt);
   PJ_LAUNCHED("k_plan_groups");
   exclusive_scan_dn<unsigned long long>(c, d.gcnt, d.qgoff, d.cap_q, nullptr, &sz->groups);
-  // A4 + A6 in one launch, then A8: the short indexed strings
+  if (passes) {  // A4: lookups, hits, candidate offsets
+    const unsigned g1 = persistent_grid(k_group_counts<false, true>, (d.cap_groups + BLOCK - 1) / BLOCK);
+    k_group_counts<false, true><<<g1, BLOCK, 0, c.stream>>>(v, d.cap_groups, d.gcounts, d.gmask, ctr, &sz->groups);
+    PJ_LAUNCHED("k_group_counts");
+    exclusive_scan_dn<uint32_t>(c, d.gcounts, d.goff, d.cap_groups, &sz->groups, &sz->hits);
+    const unsigned g2 = persistent_grid(k_group_hits<false, true>, (d.cap_groups + BLOCK - 1) / BLOCK);
+    k_group_hits<false, true><<<g2, BLOCK, 0, c.stream>>>(v, d.cap_groups, d.gcounts, d.gmask, d.goff, d.hits,
+                                                          &sz->groups, d.cap_hits);
+    PJ_LAUNCHED("k_group_hits");
+    k_hit_counts<<<stride_grid(d.cap_hits), 256, 0, c.stream>>>(d.hits, d.cap_hits, d.hcnt, &sz->hits);
+    PJ_LAUNCHED("k_hit_counts");
+    exclusive_scan_dn<unsigned long long>(c, d.hcnt, d.hoff, d.cap_hits, &sz->hits, &sz->cands);
+  }
+  // A6, without the passes A4 + A6 in one launch, then A8: the short indexed
+  // strings
   const AccOut acc{d.acc_key[0], d.acc_ed[0], d.cap_acc};
 #define PJ_CALL(W)                                                                                              \
   do {                                                                                                         \
-    launch_query<W, true>(c, v, d.cap_groups, &sz->groups, d.tasks, d.task_cap, acc, ctr);                      \
+    if (passes) {                                                                                              \
+      const unsigned gv = persistent_grid(k_verify_queued<W, false, true>, ~0ull >> 8, Q_BLOCK);                \
+      k_verify_queued<W, false, true><<<gv, Q_BLOCK, 0, c.stream>>>(v, d.hits, d.hoff, d.cap_hits, 0, 0, acc,   \
+                                                                    ctr, &sz->hits, 0);                         \
+      PJ_LAUNCHED("k_verify_queued");                                                                          \
+    } else {                                                                                                   \
+      launch_query<W, true>(c, v, d.cap_groups, &sz->groups, d.tasks, d.task_cap, acc, ctr);                    \
+    }                                                                                                          \
     if (has_short) {                                                                                           \
       const unsigned gf = persistent_grid(k_fallback<W, false, true>, (d.cap_q + BLOCK - 1) / BLOCK);           \
       k_fallback<W, false, true><<<gf, BLOCK, 0, c.stream>>>(v, d.cap_q, acc, ctr, &sz->n);                     \
@@ -3764,7 +3782,7 @@ void record_query_plan(const Ctx& c, const pj_index& idx, const PlanDev& d) {
   k_emit_pairs<<<stride_grid(d.cap_acc), 256, 0, c.stream>>>(keys, eds, d.flags, d.pos, d.cap_acc, v.key_shift,
                                                              d.out_pairs, &ctr->accepted, d.cap_pairs);
   PJ_LAUNCHED("k_emit_pairs");
-  k_plan_finish<<<1, 1, 0, c.stream>>>(ctr, sz, d.header);
+  k_plan_finish<<<1, 1, 0, c.stream>>>(ctr, sz, passes, d.header);
   PJ_LAUNCHED("k_plan_finish");
 }
 

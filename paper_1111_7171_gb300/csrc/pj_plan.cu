@@ -40,31 +40,51 @@ struct pj_plan {
   pj::DBuf<pj::Planes> planes;
   pj::DBuf<pj::PartView> parts;
   pj::DBuf<pj::Hit> tasks;
+  // the probe passes' state (empty: not recorded)
+  pj::DBuf<uint32_t> gcounts, goff;
+  pj::DBuf<unsigned long long> gmask, hcnt, hoff;
+  pj::DBuf<pj::Hit> hits;
   pj::DBuf<unsigned char> counters, arena;
   // pinned host buffers
   pj::HostBuf h_bytes, h_off, h_tau, h_n, h_pairs, h_header;
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
-  uint32_t nodes = 0, kernels = 0;
+  // the pipeline with the query kernel, and with the probe passes
+  struct Graph {
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    uint32_t nodes = 0, kernels = 0;
+    void drop() {
+      if (exec) cudaGraphExecDestroy(exec);
+      if (graph) cudaGraphDestroy(graph);
+      *this = Graph{};
+    }
+  };
+  Graph graphs[2];
+  int last = 0;  // the one that ran last
   uint64_t runs = 0, captures = 0;
 
   uint64_t device_bytes() const {
-    return bytes.bytes() + tau.bytes() + off.bytes() + sizes.bytes() + len.bytes() + flags.bytes() + pos.bytes() + acc_ed0.bytes() + acc_ed1.bytes() + gcnt.bytes() + qgoff.bytes() +
-           bm.bytes() + planes.bytes() + acc_key0.bytes() + acc_key1.bytes() + parts.bytes() + counters.bytes() +
-           arena.bytes() + tasks.bytes();
+    return bytes.bytes() + tau.bytes() + off.bytes() + sizes.bytes() + len.bytes() + flags.bytes() + pos.bytes() +
+           acc_ed0.bytes() + acc_ed1.bytes() + gcnt.bytes() + qgoff.bytes() + bm.bytes() + planes.bytes() +
+           acc_key0.bytes() + acc_key1.bytes() + parts.bytes() + counters.bytes() + arena.bytes() + tasks.bytes() +
+           gcounts.bytes() + goff.bytes() + gmask.bytes() + hcnt.bytes() + hoff.bytes() + hits.bytes();
   }
   uint64_t host_bytes() const {
     return h_bytes.bytes + h_off.bytes + h_tau.bytes + h_n.bytes + h_pairs.bytes + h_header.bytes;
   }
-  void drop_graph() {
-    if (exec) cudaGraphExecDestroy(exec);
-    if (graph) cudaGraphDestroy(graph);
-    exec = nullptr;
-    graph = nullptr;
+  void drop_graphs() {
+    for (Graph& g : graphs) g.drop();
+  }
+  void release_passes() {
+    gcounts.release();
+    goff.release();
+    gmask.release();
+    hits.release();
+    hcnt.release();
+    hoff.release();
   }
   void release_all() {
     if (stream) cudaStreamSynchronize(stream);  // nothing of the plan in flight
-    drop_graph();
+    drop_graphs();
     pj::DBuf<uint8_t>* b8[] = {&bytes, &tau};
     for (auto* b : b8) b->release();
     off.release();
@@ -77,6 +97,7 @@ struct pj_plan {
     planes.release();
     parts.release();
     tasks.release();
+    release_passes();
     counters.release();
     arena.release();
     if (stream) cudaStreamSynchronize(stream);
@@ -95,6 +116,19 @@ namespace {
 constexpr unsigned long long MAX_CAP_ACC = 0xFFFFFFFFull;  // radix sort and u32 positions
 
 // (Re)allocate the capacity-dependent buffers for d's capacities.
+bool alloc_hits(pj_plan& P) {
+  const bool ok = P.hits.try_reset(P.ctx, P.d.cap_hits) && P.hcnt.try_reset(P.ctx, P.d.cap_hits) &&
+                  P.hoff.try_reset(P.ctx, P.d.cap_hits);
+  if (!ok) P.release_passes();  // batches of any size then run in one launch
+  P.d.gcounts = P.gcounts.p;
+  P.d.goff = P.goff.p;
+  P.d.gmask = P.gmask.p;
+  P.d.hits = P.hits.p;
+  P.d.hcnt = P.hcnt.p;
+  P.d.hoff = P.hoff.p;
+  return ok;
+}
+
 void alloc_acc(pj_plan& P) {
   P.acc_key0.reset(P.ctx, P.d.cap_acc);
   P.acc_key1.reset(P.ctx, P.d.cap_acc);
@@ -115,68 +149,77 @@ void alloc_pairs(pj_plan& P) {
   P.d.out_pairs = static_cast<pj_pair*>(P.h_pairs.dev);
 }
 
-// Records the pipeline into a fresh graph and instantiates it.
+// Records the pipeline into a fresh graph and instantiates it; false when the
+// arena is too small.  Both graphs have their temporaries in the same arena,
+// since one of them runs at a time.
+bool capture_one(pj_plan& P, bool passes) {
+  pj_plan::Graph& G = P.graphs[passes];
+  G.drop();
+  Arena ar;
+  ar.base = P.arena.p;
+  ar.cap = P.arena.bytes();
+  Ctx rc;
+  rc.stream = P.stream;
+  rc.alloc = arena_alloc;
+  rc.free_fn = arena_free;
+  rc.alloc_ctx = &ar;
+  cudaGraph_t g = nullptr;
+  PJ_CUDA(cudaStreamBeginCapture(P.stream, cudaStreamCaptureModeRelaxed));
+  set_recording(true);
+  bool ok = true;
+  Error err{PJ_OK, ""};
+  try {
+    record_query_plan(rc, *P.idx, P.d, passes);
+  } catch (const Error& e) {
+    ok = false;
+    err = e;
+  }
+  set_recording(false);
+  const cudaError_t ce = cudaStreamEndCapture(P.stream, &g);
+  if (!ok || ce != cudaSuccess || !g) {
+    if (g) cudaGraphDestroy(g);
+    cudaGetLastError();
+    if (!ok && ar.exhausted) return false;
+    if (!ok) throw err;
+    fail(PJ_ECUDA, std::string("query plan: graph capture failed: ") + cudaGetErrorString(ce));
+  }
+  G.graph = g;
+  const cudaError_t ie = cudaGraphInstantiate(&G.exec, g, 0);
+  if (ie != cudaSuccess) {
+    cudaGetLastError();
+    G.exec = nullptr;
+    G.drop();
+    fail(PJ_ECUDA, std::string("query plan: cudaGraphInstantiate failed: ") + cudaGetErrorString(ie));
+  }
+  size_t n = 0;
+  PJ_CUDA(cudaGraphGetNodes(g, nullptr, &n));
+  std::vector<cudaGraphNode_t> nodes(n);
+  PJ_CUDA(cudaGraphGetNodes(g, nodes.data(), &n));
+  uint32_t kernels = 0;
+  for (size_t k = 0; k < n; ++k) {
+    cudaGraphNodeType t;
+    PJ_CUDA(cudaGraphNodeGetType(nodes[k], &t));
+    if (t == cudaGraphNodeTypeKernel) ++kernels;
+  }
+  G.nodes = (uint32_t)n;
+  G.kernels = kernels;
+  return true;
+}
+
+// Records the plan's graphs.
 void capture(pj_plan& P) {
-  P.drop_graph();
+  P.drop_graphs();
   size_t arena_bytes = scan_temp_bytes(P.d.cap_q) + scan_temp_bytes(P.d.cap_acc) +
                        sort_temp_bytes(P.d.cap_acc) + (1u << 16);
+  if (P.d.hits) arena_bytes += scan_temp_bytes(P.d.cap_groups) + scan_temp_bytes(P.d.cap_hits);
   for (int attempt = 0;; ++attempt) {
     P.arena.reset(P.ctx, arena_bytes);
     P.ctx.sync();
-    Arena ar;
-    ar.base = P.arena.p;
-    ar.cap = arena_bytes;
-    Ctx rc;
-    rc.stream = P.stream;
-    rc.alloc = arena_alloc;
-    rc.free_fn = arena_free;
-    rc.alloc_ctx = &ar;
-    cudaGraph_t g = nullptr;
-    PJ_CUDA(cudaStreamBeginCapture(P.stream, cudaStreamCaptureModeRelaxed));
-    set_recording(true);
-    bool ok = true;
-    Error err{PJ_OK, ""};
-    try {
-      record_query_plan(rc, *P.idx, P.d);
-    } catch (const Error& e) {
-      ok = false;
-      err = e;
-    }
-    set_recording(false);
-    const cudaError_t ce = cudaStreamEndCapture(P.stream, &g);
-    if (!ok || ce != cudaSuccess || !g) {
-      if (g) cudaGraphDestroy(g);
-      cudaGetLastError();
-      if (!ok && ar.exhausted && attempt < 4) {  // the estimate was short: retry with more
-        arena_bytes *= 2;
-        continue;
-      }
-      if (!ok) throw err;
-      fail(PJ_ECUDA, std::string("query plan: graph capture failed: ") + cudaGetErrorString(ce));
-    }
-    P.graph = g;
-    const cudaError_t ie = cudaGraphInstantiate(&P.exec, g, 0);
-    if (ie != cudaSuccess) {
-      cudaGetLastError();
-      P.exec = nullptr;
-      P.drop_graph();
-      fail(PJ_ECUDA, std::string("query plan: cudaGraphInstantiate failed: ") + cudaGetErrorString(ie));
-    }
-    size_t n = 0;
-    PJ_CUDA(cudaGraphGetNodes(g, nullptr, &n));
-    std::vector<cudaGraphNode_t> nodes(n);
-    PJ_CUDA(cudaGraphGetNodes(g, nodes.data(), &n));
-    uint32_t kernels = 0;
-    for (size_t k = 0; k < n; ++k) {
-      cudaGraphNodeType t;
-      PJ_CUDA(cudaGraphNodeGetType(nodes[k], &t));
-      if (t == cudaGraphNodeTypeKernel) ++kernels;
-    }
-    P.nodes = (uint32_t)n;
-    P.kernels = kernels;
-    ++P.captures;
-    return;
+    if (capture_one(P, false) && (!P.d.hits || capture_one(P, true))) break;
+    if (attempt >= 4) fail(PJ_ENOMEM, "query plan: temporaries outgrow their estimate");
+    arena_bytes *= 2;  // the estimate was short: retry with more
   }
+  ++P.captures;
 }
 
 uint64_t grown(uint64_t cap, uint64_t need, uint64_t limit, const char* what) {
@@ -208,8 +251,9 @@ void create(pj_plan& P, pj_index& idx, const pj_plan_options& o) {
   PlanDev& d = P.d;
   d.cap_q = o.max_queries;
   d.cap_groups = cap_groups;
-  // hits take no room since the query kernel keeps none; the capacity only
-  // bounds what a batch may find before the plan is recorded again, as before.
+  // hits take no room in the query kernel, only in the probe passes; without
+  // those the capacity bounds what a batch may find before the plan is recorded
+  // again.
   // defaults: about two hits per group and 128 accepted matches per query
   // (the short-string workload at tau = 4 averages 1.7 and 217 at full
   // self-join scale); capacities grow when a batch needs more
@@ -231,7 +275,19 @@ void create(pj_plan& P, pj_index& idx, const pj_plan_options& o) {
   P.gcnt.reset(P.ctx, d.cap_q);
   P.qgoff.reset(P.ctx, d.cap_q);
   P.counters.reset(P.ctx, PLAN_COUNTER_BYTES);
-  d.task_cap = query_task_room(cap_groups, idx.n);
+  // Batches of more than QUERY_FUSED_MAX_GROUPS take the probe passes against
+  // short strings.  Passes / query kernel, mixed thresholds up to 4, ms: 16,384
+  // queries against 300k strings 1.00 / 1.21, 65,536 3.16 / 3.78, against 1M
+  // strings 2.19 / 2.24 and 9.1 / 9.0; up to 3, 65,536 against 1M 2.16 / 2.29.
+  // Longer strings have few candidates and stay with the query kernel: 8,192
+  // queries of titles at thresholds up to 8 take 0.74 ms with it, 2.1 ms with
+  // the passes.
+  if (idx.splanes.p && cap_groups > QUERY_FUSED_MAX_GROUPS && P.gcounts.try_reset(P.ctx, cap_groups) &&
+      P.goff.try_reset(P.ctx, cap_groups) && P.gmask.try_reset(P.ctx, cap_groups))
+    alloc_hits(P);
+  else
+    P.release_passes();
+  d.task_cap = query_task_room(d.hits ? QUERY_FUSED_MAX_GROUPS : cap_groups, idx.n);
   while (d.task_cap && !P.tasks.try_reset(P.ctx, d.task_cap))  // without any, long runs stay with their warps
     d.task_cap = d.task_cap > (1u << 12) ? d.task_cap / 2 : 0;
   d.tasks = P.tasks.p;
@@ -286,11 +342,13 @@ void plan_query(pj_plan& P, const pj_strings& b, const uint8_t* taus, pj_result*
   // validate and stage the batch (offsets rebased to 0)
   const uint64_t base = b.offsets[0];
   uint64_t* hoff = static_cast<uint64_t*>(P.h_off.p);
+  uint64_t groups = 0;
   for (uint32_t q = 0; q < n; ++q) {
     if (b.offsets[q + 1] < b.offsets[q] || b.offsets[q + 1] - b.offsets[q] > 65535)
       fail(PJ_EINVAL, "pj_strings: offsets decrease or a string is longer than 65535 bytes");
     if ((int)taus[q] > tau_max) fail(PJ_EINVAL, "pj_plan_query: tau outside 0..tau_max");
     hoff[q] = b.offsets[q] - base;
+    groups += (uint64_t)groups_per_probe((int)taus[q], false);
   }
   const uint64_t total = b.offsets[n] - base;
   hoff[n] = total;
@@ -307,8 +365,9 @@ void plan_query(pj_plan& P, const pj_strings& b, const uint8_t* taus, pj_result*
 
   PlanHeader h{};
   for (int attempt = 0;; ++attempt) {
-    PJ_CUDA(cudaGraphLaunch(P.exec, P.stream));
-    count_launches(P.kernels);
+    P.last = P.d.hits && groups > QUERY_FUSED_MAX_GROUPS;
+    PJ_CUDA(cudaGraphLaunch(P.graphs[P.last].exec, P.stream));
+    count_launches(P.graphs[P.last].kernels);
     P.ctx.sync();
     ++P.runs;
     memcpy(&h, P.h_header.p, sizeof(h));
@@ -319,6 +378,7 @@ void plan_query(pj_plan& P, const pj_strings& b, const uint8_t* taus, pj_result*
     if (short_of_room && attempt >= 8) fail(PJ_ECUDA, "query plan: capacities still too small after growing");
     if (h.hits > P.d.cap_hits) {
       P.d.cap_hits = grown(P.d.cap_hits, h.hits, P.d.cap_groups * (uint64_t)(tau_max + 1), "hits");
+      if (P.d.hits) alloc_hits(P);
     } else if (h.accepted > P.d.cap_acc) {
       P.d.cap_acc = grown(P.d.cap_acc, h.accepted, MAX_CAP_ACC, "accepted matches");
       alloc_acc(P);
@@ -417,8 +477,8 @@ int pj_plan_get_info(const pj_plan* plan, pj_plan_info* out) {
   memset(out, 0, sizeof(*out));
   out->runs = P->runs;
   out->recaptures = P->captures ? P->captures - 1 : 0;
-  out->graph_nodes = P->nodes;
-  out->graph_kernels = P->kernels;
+  out->graph_nodes = P->graphs[P->last].nodes;
+  out->graph_kernels = P->graphs[P->last].kernels;
   out->hits_capacity = P->d.cap_hits;
   out->accepted_capacity = P->d.cap_acc;
   out->pairs_capacity = P->d.cap_pairs;

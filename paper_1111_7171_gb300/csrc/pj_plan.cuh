@@ -51,6 +51,13 @@ struct PlanDev {
   void* counters;                 // PLAN_COUNTER_BYTES, zeroed by the graph
   Hit* tasks;                     // task_cap parts of long posting runs
   unsigned long long task_cap;
+  // the probe passes of large batches (NULL: not recorded)
+  uint32_t* gcounts;              // cap_groups
+  uint32_t* goff;                 // cap_groups
+  unsigned long long* gmask;      // cap_groups window-position masks
+  Hit* hits;                      // cap_hits
+  unsigned long long* hcnt;       // cap_hits
+  unsigned long long* hoff;       // cap_hits
   unsigned long long* acc_key[2]; // cap_acc each (sort double buffer)
   uint32_t* acc_ed[2];
   uint32_t* flags;                // cap_acc
@@ -122,6 +129,11 @@ inline size_t sort_temp_bytes(size_t n) {
   return align256(8 * (RS_HIST_WORDS + 8 * 256 * ((n + RS_TILE - 1) / RS_TILE)));
 }
 
+// Groups up to which a query batch runs in one launch (k_query_fused); a larger
+// R != S join takes the probe passes, whose lanes roll a window's keys, and so
+// does a plan's batch against an index of short strings.
+constexpr unsigned long long QUERY_FUSED_MAX_GROUPS = 1ull << 18;
+
 // Room for the parts of long runs that a batch of `groups` groups sets aside
 // (k_query_fused, 32 bytes each): 2^12 for small batches, at most 256 MiB.  A
 // million short strings have between 1.4 and 2.7 parts a group at tau <= 4, and
@@ -137,6 +149,6 @@ inline unsigned long long query_task_room(unsigned long long groups, uint32_t n_
 // Enqueues the whole query pipeline for the buffers in d on c's stream
 // without any host synchronisation (meant to run under stream capture).
 // Temporaries come from c's allocator and must outlive the recorded work.
-void record_query_plan(const Ctx& c, const pj_index& idx, const PlanDev& d);
+void record_query_plan(const Ctx& c, const pj_index& idx, const PlanDev& d, bool passes);
 
 }  // namespace pj

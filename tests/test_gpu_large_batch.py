@@ -1,6 +1,8 @@
 """Plans of many queries: room for the parts of long posting runs grows with
 the batch (without it most runs are walked unevenly, by the warps that found
-them)."""
+them), and batches of more than 2^18 groups are answered by the probe passes
+where the strings are short."""
+import numpy as np
 import pytest
 
 from paper_1111_7171_gb300 import passjoin as pj
@@ -20,4 +22,30 @@ def test_plan_has_room_for_four_parts_a_group():
     assert more >= PART_BYTES * (4 * groups * 5_000 - 4096)
     small.free()
     large.free()
+    idx.free()
+
+
+@pytest.mark.parametrize("hits_capacity", [0, 1])
+def test_large_batches_take_the_probe_passes(hits_capacity):
+    strings = synth.generate("short", 4, n=20_000) + [b"", b"ab", b"abcd"]
+    idx = pj.pj_build_index(strings, 4)
+    queries = [s[1:] + s[:1] for s in strings[:16_000]]
+    taus = (np.arange(len(queries)) % 5).astype(np.uint8)  # 19 groups on average, 304,000 in all
+    plan = pj.Plan(idx, max_queries=16_384, max_bytes=1 << 20, hits_capacity=hits_capacity)
+    got = plan.query(queries, taus)
+    passes = plan.info()["graph_kernels"]
+    q = len(queries) // 4
+    lookups = hits = 0
+    for k in range(4):  # in quarters, eager: the query kernel
+        want = pj.pj_query_multi(idx, queries[k * q:(k + 1) * q], taus[k * q:(k + 1) * q])
+        lookups, hits = lookups + want.stats["lookups"], hits + want.stats["hits"]
+        part = got.pairs[(got.pairs["a"] >= k * q) & (got.pairs["a"] < (k + 1) * q)].copy()
+        part["a"] -= k * q
+        assert np.array_equal(part, want.pairs)
+        assert np.array_equal(plan.query(queries[k * q:(k + 1) * q], taus[k * q:(k + 1) * q]).pairs, want.pairs)
+        assert plan.info()["graph_kernels"] < passes
+    assert (got.stats["lookups"], got.stats["hits"]) == (lookups, hits)
+    again = plan.query(queries, taus)
+    assert np.array_equal(again.pairs, got.pairs) and plan.info()["graph_kernels"] == passes
+    plan.free()
     idx.free()
