@@ -5,8 +5,11 @@ where the strings are short."""
 import numpy as np
 import pytest
 
+pytest.importorskip("torch")
+
 from paper_1111_7171_gb300 import passjoin as pj
 from paper_1111_7171_gb300 import synth
+from test_gpu_tight_memory import Memory
 
 pytestmark = pytest.mark.gpu
 
@@ -49,3 +52,21 @@ def test_large_batches_take_the_probe_passes(hits_capacity):
     assert np.array_equal(again.pairs, got.pairs) and plan.info()["graph_kernels"] == passes
     plan.free()
     idx.free()
+
+
+@pytest.mark.parametrize("refused", [4 * 45 * 16_384, 8 * 45 * 16_384, 32 * 2 * 45 * 16_384, 32 << 20])
+def test_large_plans_without_memory(refused, monkeypatch):
+    """Group counts, masks, hits (32 bytes, two a group) or the parts' room
+    refused once: the plan does without, or with less room."""
+    strings = synth.generate("short", 4, n=20_000)
+    mem = Memory(monkeypatch)
+    idx = pj.pj_build_index(strings, 4)
+    queries, taus = strings[:16_000], (np.arange(16_000) % 5).astype(np.uint8)
+    want = pj.pj_query_multi(idx, queries, taus).pairs
+    mem.refused, mem.refusals = [refused], 0
+    plan = pj.Plan(idx, max_queries=16_384, max_bytes=1 << 20)
+    assert mem.refusals == 1
+    assert np.array_equal(plan.query(queries, taus).pairs, want)
+    plan.free()
+    idx.free()
+    assert mem.now == 0
