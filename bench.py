@@ -49,14 +49,19 @@ METRIC = "self-join verified similar pairs/s"
 UNIT = "pairs/s"
 L2_FLUSH_BYTES = 256 << 20
 OPS_PER_CELL = 6            # integer ops of one DP cell: delta compare, diagonal add, up/left +1, two mins
-SCREEN_BYTES = 16           # one posting record (sid + character signature) read per candidate
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of k_verify_queued
-# over one self join of the short workload at 1,000,000 strings and tau 4, from
-# a one-pass ncu capture of the current kernel: the join's short first launch
-# (0.022 GB read, 1.244 GB written: mostly the write-back of the hits written
-# just before it) and its one long launch (4.343 GB read, 1.310 GB written).
-# The 16-byte posting records the join screens (356 GB) are read from L2.
-VERIFY_TRAFFIC_SHORT1M_TAU4 = (0.022 + 1.244 + 4.343 + 1.310) * 1e9
+SCREEN_BYTES = 16           # one posting record (sid + character counts) read per candidate
+# integer instructions of one candidate of the tiles' screen (k_screen_tiles):
+# six byte distances, two limit compares and the run compare, one for the ballot
+TILE_SCREEN_OPS = 10
+# joins that the library verifies by tiles (TILES_MIN_HITS, TILES_MIN_RUN in
+# csrc/pj_join.cu)
+TILES_MIN_HITS, TILES_MIN_RUN = 1 << 20, 60
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of k_screen_tiles
+# and k_verify_list over one self join of the short workload at 1,000,000
+# strings and tau 4, from a one-pass ncu capture of the current kernels: the
+# screen's 1.859 GB read and 29.612 GB written (the survivors' list), the
+# verification's 23.912 GB read and 2.502 GB written.
+VERIFY_TRAFFIC_SHORT1M_TAU4 = (1.859 + 29.612 + 23.912 + 2.502) * 1e9
 
 
 def parse():
@@ -552,36 +557,48 @@ def run_native(args):
         # candidates that reach a DP: those the character-count screen keeps
         # (mode L: the distinct pairs it keeps)
         dp_verified = (st["distinct_pairs"] if pair_mode else st["candidates"]) - st["filtered"]
-        kernel = ("k_verify_pairs_warp" if st["pair_warp"] else "k_verify_pairs") if pair_mode else "k_verify_queued"
+        tiled = (not pair_mode and not st["fused"] and st["hits"] >= TILES_MIN_HITS
+                 and st["candidates"] >= TILES_MIN_RUN * st["hits"])
+        kernel = ("k_verify_pairs_warp" if st["pair_warp"] else "k_verify_pairs") if pair_mode else \
+            "k_screen_tiles + k_verify_list" if tiled else "k_verify_queued"
         if st["fused"]:  # one kernel from selection to verification: its time is the verify phase
             kernel = "k_fused_self"
         alu_peak_gcells = cal["dp_cells_per_s"] / 1e9
         sm_max = float(peaks.get("sm_max_mhz", 2070.0))
         derived_gcells = cal["sm_count"] * 128 * sm_max * 1e6 / OPS_PER_CELL / 1e9
         achieved = cells / (verify_ms / 1e3) / 1e9
-        headline = (args.workload == "short" and n == 1_000_000 and args.tau == 4 and kernel == "k_verify_queued")
+        headline = args.workload == "short" and n == 1_000_000 and args.tau == 4 and tiled
         traffic = VERIFY_TRAFFIC_SHORT1M_TAU4 if headline else None
         roofline = {"bound": "alu", "kernel": kernel, "achieved": achieved, "peak": alu_peak_gcells,
                     "unit": "Gcell/s", "frac": achieved / alu_peak_gcells, "traffic": traffic,
-                    "traffic_unit": ("DRAM bytes of the verification kernel per join, both launches (ncu "
+                    "traffic_unit": ("DRAM bytes of the screen and verification kernels per join, all launches (ncu "
                                      "dram__bytes_read.sum + dram__bytes_write.sum), like `achieved`, which is per "
-                                     "second of the join's verification; its algorithmic record stream is "
-                                     f"{cands * SCREEN_BYTES / 1e9:.0f} GB, read from L2") if headline else None,
-                    "work": "DP cells evaluated by the verification (counted exactly), per second of verification",
+                                     "second of the join's verification") if headline else None,
+                    "work": "DP cells evaluated by the verification (counted exactly; on bit planes, short strings, "
+                            "furthest-reaching cells, T + 1 an edit), per second of verification, screen included",
                     "peak_source": f"measured (pj_calibrate): the verification's banded cell recurrence with "
                                    f"operands in registers, {alu_peak_gcells:.0f} Gcell/s at {cal['sm_mhz']:.0f} MHz "
                                    f"on {cal['sm_count']} SMs (unit count x clock: {cal['sm_count']} SMs x 128 "
                                    f"int32 lanes x {sm_max:.0f} MHz / {OPS_PER_CELL} ops per cell = "
                                    f"{derived_gcells:.0f} Gcell/s; measured int32 rate "
                                    f"{cal['int32_ops_per_s'] / 1e12:.1f} Tops/s)"}
-        screen_bytes = (st["distinct_pairs"] if pair_mode else cands) * SCREEN_BYTES
-        screen_gbs = screen_bytes / (verify_ms / 1e3) / 1e9
-        roofline_screen = {"bound": "l2", "kernel": kernel, "achieved": screen_gbs,
-                           "peak": cal["l2_read_bytes_per_s"] / 1e9, "unit": "GB/s",
-                           "frac": screen_gbs / (cal["l2_read_bytes_per_s"] / 1e9),
-                           "work": f"{SCREEN_BYTES} B posting record per candidate screened, per second of "
-                                   "verification",
-                           "peak_source": "measured (pj_calibrate): 16-byte loads over a 64 MiB L2-resident buffer"}
+        if tiled:  # a record stays in registers for up to 256 hits of its run: bound by instructions
+            screen_ops = cands * TILE_SCREEN_OPS / (verify_ms / 1e3)
+            roofline_screen = {"bound": "alu", "kernel": "k_screen_tiles", "achieved": screen_ops / 1e9,
+                               "peak": cal["int32_ops_per_s"] / 1e9, "unit": "Gop/s",
+                               "frac": screen_ops / cal["int32_ops_per_s"],
+                               "work": f"{TILE_SCREEN_OPS} integer instructions per candidate screened, per second "
+                                       "of verification (screen and verification kernels)",
+                               "peak_source": "measured (pj_calibrate): independent xor + add chains"}
+        else:
+            screen_bytes = (st["distinct_pairs"] if pair_mode else cands) * SCREEN_BYTES
+            screen_gbs = screen_bytes / (verify_ms / 1e3) / 1e9
+            roofline_screen = {"bound": "l2", "kernel": kernel, "achieved": screen_gbs,
+                               "peak": cal["l2_read_bytes_per_s"] / 1e9, "unit": "GB/s",
+                               "frac": screen_gbs / (cal["l2_read_bytes_per_s"] / 1e9),
+                               "work": f"{SCREEN_BYTES} B posting record per candidate screened, per second of "
+                                       "verification",
+                               "peak_source": "measured (pj_calibrate): 16-byte loads over a 64 MiB L2-resident buffer"}
         serving = None
         if not args.no_serve and args.workload == "short":
             serving = serving_bench(strings, args.serve_requests)
@@ -620,7 +637,8 @@ def run_native(args):
                     "h2d_bytes_per_step": int(buf.nbytes + off.nbytes),
                     "d2h_bytes_per_step": int(e2e_pairs * 12)},
             "resident_join": dict(resident, note="join alone on a resident index, mean over the timed steps; "
-                                                 "graph = one recorded CUDA graph replayed per join; eager/graph "
+                                                 "graph = one recorded CUDA graph replayed per join (graph_replays "
+                                                 "0: verified by tiles, which stays eager); eager/graph "
                                                  "use the tuned form (choice), chunked_* the chunked pipeline, "
                                                  "fused_* the fused kernel with a thread / a warp per pair"),
             "gpu_launches": int(launches),

@@ -101,7 +101,8 @@ typedef struct {
   uint64_t lookups;     /* selected substrings looked up in the segment index */
   uint64_t candidates;  /* (probe, indexed string, segment, position) matches verified */
   uint64_t accepted;    /* matches accepted by extension verification */
-  uint64_t dp_cells;    /* DP cells evaluated by the verification kernels */
+  uint64_t dp_cells;    /* DP cells evaluated by the verification kernels (on bit planes, where the
+                           strings have them: furthest-reaching cells, T + 1 for every edit tried) */
   uint64_t fallback_pairs; /* pairs verified directly because a string has length <= tau */
   uint64_t hits;        /* lookups whose posting run was non-empty */
   float probe_ms;       /* device time of selection + lookup (CUDA events on the call's stream); 0 for a

@@ -47,11 +47,14 @@ namespace cg = cooperative_groups;
 
 constexpr int BLOCK = 256;
 
-// The kernels of this file use no warp-level collectives and no block
-// barriers: every thread works alone and publishes through global atomics or
-// prefix sums.  (Earlier forms that placed shuffles, ballots or
-// __syncthreads right after the divergent verification loops lost the
-// contributions of lanes still inside those loops.)
+// The thread-per-item kernels of this file use no warp collectives inside
+// their divergent loops and no block barriers: every thread works alone and
+// publishes through global atomics or prefix sums.  Their counters are added
+// by warps at the end, after a __syncwarp that brings back the lanes still
+// inside the loops (warp_add_counter; earlier forms with shuffles, ballots or
+// __syncthreads right after such loops and without it lost those lanes'
+// contributions).  The warp kernels reconverge in the same way before each
+// ballot.
 
 // ---------------------------------------------------------------- A4 ------
 
@@ -373,8 +376,10 @@ __global__ void __launch_bounds__(512) k_verify_hits(const ProbeView v, const Hi
 // Q_CHUNK, times up to 4 when every warp gets at least 512 chunks of that
 // size (measured on 2.2e10 candidates: 3% less time with 4; on 3e8, where a
 // warp gets 30 chunks, larger chunks unbalance the warps), and in launches
-// that have less than a chunk for every warp an even share, so that a small
-// batch does not leave most of the GPU idle (64 queries: 162 -> 45 us).
+// that have less than a chunk for every warp an even share, so that a launch
+// of few candidates does not leave most of the GPU idle (a batch of 4,096
+// queries of titles at thresholds up to 8, whose probe passes end here: 11.3 ms
+// with a chunk of 2,048 throughout, 2.0 ms now).
 __host__ __device__ __forceinline__ unsigned long long queued_chunk(unsigned long long n, unsigned long long n_warps) {
   const unsigned long long share = n / n_warps;
   if (share >= 512 * Q_CHUNK) return Q_CHUNK * ::min(4ull, share / (512 * Q_CHUNK));
@@ -1617,10 +1622,20 @@ static void launch_verify(const Ctx& c, const ProbeView& v, const Hit* hits, con
 
 // Hits, and candidates per hit, from which a chunk is grouped by run and
 // verified tile by tile (PJ_TILES_MIN_HITS overrides the first and drops the
-// second).  Probe + verification, tiles / queued, by candidates per hit: 27
-// (417k short strings, tau 2) 1.39 / 1.25 ms, 50 (200k, tau 3) 1.82 / 1.95, 54
-// (1M, tau 2) 3.22 / 2.93, 64 (100k, tau 4) 1.93 / 2.30, 92 (417k, tau 3) 4.3 /
-// 5.4, 521 (1M, tau 4) 95 / 138 ms.
+// second).  Probe + verification of short strings, tiles / queued, ms, by
+// threshold, with millions of hits and candidates per hit:
+//   tau 2:  1.0, 18 (250k strings) 0.81 / 0.72; 1.9, 27 (417k) 1.21 / 1.05; 5.4, 54
+//     (1M) 2.99 / 2.80; 6.7, 62 (1.2M) 3.77 / 3.72; 8.0, 70 (1.4M) 4.39 / 4.57;
+//     12, 96 (2M) 7.0 / 8.2
+//   tau 3:  0.3, 11 (30k) 0.45 / 0.31; 0.7, 19 (60k) 0.58 / 0.60; 1.4, 28 (100k)
+//     0.80 / 0.90; 2.2, 39 (150k) 1.21 / 1.20; 3.1, 49 (200k) 1.61 / 1.73; 6.9, 90
+//     (400k) 3.68 / 4.75
+//   tau 4:  0.2, 10 (10k) 0.40 / 0.22; 0.6, 16 (20k) 0.51 / 0.42; 1.3, 29 (40k)
+//     0.68 / 0.71; 2.0, 40 (60k) 0.98 / 1.00; 3.5, 63 (100k) 1.67 / 2.09; 7.7, 116
+//     (200k) 4.4 / 6.6
+// Grouping costs some 0.2 ms whatever the hits, and pays by the candidates: at
+// 60 a hit it is ahead, or even at tau 2, at every threshold; below, between 0.2
+// ms behind and 10% ahead.  2^20 hits keep the fixed cost below a quarter.
 constexpr unsigned long long TILES_MIN_HITS = 1ull << 20;
 constexpr unsigned long long TILES_MIN_RUN = 60;
 
@@ -1795,7 +1810,8 @@ static void pinned_put(void* p, size_t bytes) {
 //   PJ_LAUNCH_CANDS      candidates per verification launch (default 1 Gi)
 //   PJ_ACCEPT_INITIAL    initial accepted-match capacity  (default 4 Mi)
 //   PJ_GRAPH_MAX_GROUPS  groups of a recorded self join   (default 256 Mi)
-//   PJ_TILES_MIN_HITS    hits grouped by run              (default 64 Ki)
+//   PJ_TILES_MIN_HITS    hits grouped by run              (default 1 Mi, and 60
+//                        candidates a hit; see TILES_MIN_HITS)
 //   PJ_GRAPH_TIGHT       1: record self joins with half their counts as
 //                        capacities, so that every replay overflows
 static unsigned long long env_knob(const char* name, unsigned long long dflt) {

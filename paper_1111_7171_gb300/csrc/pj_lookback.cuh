@@ -1,5 +1,5 @@
-// Decoupled look-back: the running sum over the tiles before a tile, found
-// while those tiles are still at work.  A tile's status word holds its own
+// Decoupled look-back (D. Merrill and M. Garland, 2016): the running sum over
+// the tiles before a tile, found while those tiles are still at work.  A tile's status word holds its own
 // sum as soon as it is known, and later the sum over all tiles up to it.
 // Word: 2 flag bits on top, the value below; written and read as one 64-bit
 // access, so flag and value always belong together.  The words are zero

@@ -20,6 +20,11 @@
 // items are sorted by one block that keeps them in shared memory over all
 // passes.
 //
+// The methods: look-back after D. Merrill and M. Garland, "Single-pass
+// Parallel Prefix Scan with Decoupled Look-back" (2016); one counting kernel
+// and one look-back per pass after A. Adinets and D. Merrill, "Onesweep: A
+// Faster Least Significant Digit Radix Sort for GPUs" (2022).
+//
 // What bounds it: the ranking's instructions and the look-back's loads, not
 // HBM (1.6 ms per pass over 2.17e8 8-byte keys, 0.52 ms of it by bytes).
 // Ballots, because match.any takes 260 cycles per warp for random 8-bit
